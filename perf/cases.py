@@ -329,6 +329,146 @@ def run(s):
     return [p.outputs(c) for p in s.projections.values()]
 
 
+# ---- the same results in 64 bits ---------------------------------------------------------------------
+class _Mixed64:
+    """`X W + s (X A^T) B` per row of one batch, its gradients and the update, in torch float64."""
+
+    def __init__(self, c, seed):
+        segs, self.rows = _segments(c, seed)
+        self.first = self.rows - c["tune_rows"]                     # fine-tuning rows are the last ones, in save order
+        row_adapter = np.full(self.rows, -1)
+        for start, n, a, _ in segs:
+            row_adapter[start:start + n] = a
+        self.sequences = [(int(s), int(n)) for s, n, _, _ in segs if n > 0]
+        self.row_adapter = row_adapter
+        self.slots = list(dict.fromkeys(int(a) for _, n, a, flag in segs if flag and n > 0))
+        self.keep = None
+        if c["dropout"]:
+            self.keep = _kept(int(seed), c["tune_rows"], c["d_in"], c["dropout"]) / (1.0 - c["dropout"])
+
+    def groups(self, first=0, slots=None):
+        ids = self.row_adapter[first:]
+        for a in (sorted(set(ids[ids >= 0].tolist())) if slots is None else slots):
+            yield a, torch.from_numpy(np.flatnonzero(ids == a)).cuda()
+
+    def linear(self, x, W, A, B, scale, first=0):
+        """`x` holds the rows from `first` on; differentiable in x, A and B."""
+        y = x @ W
+        for a, at in self.groups(first):
+            y = y.index_add(0, at, scale[a] * ((x[at] @ A[a].T) @ B[a]))
+        return y
+
+    def projection(self, c, p):
+        W, A, B, scale, X = (t.double() for t in (p.W, p.A, p.B, p.scale, p.X))
+        f = self.first
+        branch = X.clone()
+        if self.keep is not None:
+            branch[f:] *= self.keep
+        U = X.new_zeros(self.rows, c["rank"])
+        Y = X @ W
+        for a, at in self.groups():
+            U[at] = branch[at] @ A[a].T
+            Y[at] += scale[a] * (U[at] @ B[a])
+        out = [Y]
+        if c["tune_rows"]:
+            out += [X[f:], U[f:]]
+        if c["backward"]:
+            dY = p.dY.double()
+            dX = dY @ W.T
+            dA, dB = [], []
+            for a, at in self.groups(f, self.slots):
+                V = scale[a] * (dY[at] @ B[a].T)
+                low = V @ A[a]
+                dX[at] += low if self.keep is None else low * self.keep[at]
+                dA.append(V.T @ branch[f:][at])
+                dB.append(scale[a] * (U[f:][at].T @ dY[at]))
+            out += [torch.stack(dA), torch.stack(dB), dX]
+        if c["update"]:
+            lr, b1, b2, eps, wd = 1e-3, 0.9, 0.999, 1e-8, 0.01      # the defaults of mlora_adamw_update
+            new, moments = [], []
+            for all_rows, grads in ((A, out[3]), (B, out[4])):
+                w = all_rows[self.slots]
+                m, v = (1 - b1) * grads, (1 - b2) * grads * grads
+                w = w - lr * wd * w - lr * (m / (1 - b1)) / ((v / (1 - b2)).sqrt() + eps)
+                all_rows[self.slots] = w
+                new.append(w)
+                moments.append((m, v))
+            (mA, vA), (mB, vB) = moments
+            out += [*new, mA, mB, vA, vB, A, B]
+        return out
+
+
+def _kept(seed, rows, d_in, p):
+    """The dropout mask of mlora.h: field k & 3 of output (m << 32 | k >> 2) + 1 of a SplitMix64 stream, for element (m, k)."""
+    u = np.uint64
+    with np.errstate(over="ignore"):
+        z = (np.arange(rows, dtype=u)[:, None] << u(32)) | np.arange((d_in + 3) // 4, dtype=u)[None, :]
+        z = u(seed) + (z + u(1)) * u(0x9E3779B97F4A7C15)
+        z = (z ^ (z >> u(30))) * u(0xBF58476D1CE4E5B9)
+        z = (z ^ (z >> u(27))) * u(0x94D049BB133111EB)
+        z = z ^ (z >> u(31))
+    fields = np.stack([(z >> u(16 * j)) & u(0xFFFF) for j in range(4)], axis=-1).reshape(rows, -1)[:, :d_in]
+    return torch.from_numpy((fields >= u(round(p * 65536))).astype(np.float64)).cuda()
+
+
+def _layer64(b, x, w, n_heads, n_kv, first=0):
+    """A decoder layer over the rows from `first` on: norm eps 1e-5, rotary base 500000 on halves, causal attention in a sequence."""
+    T, d = x.shape
+    dh = d // n_heads
+
+    def norm(t, g):
+        return t * torch.rsqrt((t * t).mean(-1, keepdim=True) + 1e-5) * g
+
+    def lin(name, t):
+        return b.linear(t, *(w[k + name].double() if k in ("W_", "s_") else w[k + name] for k in ("W_", "A_", "B_", "s_")), first)
+
+    seqs = [(s - first, n) for s, n in b.sequences if s >= first]
+    pos = torch.cat([torch.arange(n) for _, n in seqs]).double().cuda()
+    inv = 500000.0 ** (-torch.arange(dh // 2, device="cuda", dtype=torch.float64) * 2.0 / dh)
+    cos, sin = torch.cos(pos[:, None] * inv)[:, None], torch.sin(pos[:, None] * inv)[:, None]
+
+    def rope(t):
+        lo, hi = t[..., :dh // 2], t[..., dh // 2:]
+        return torch.cat([lo * cos - hi * sin, hi * cos + lo * sin], -1)
+
+    h1 = norm(x, w["g1"])
+    q, k, v = (lin(n, h1).view(T, -1, dh) for n in "qkv")
+    q, k = rope(q), rope(k)
+    parts = []
+    for s, n in seqs:                                              # in row order: every row is in one sequence
+        qs, ks, vs = (t[s:s + n].transpose(0, 1) for t in (q, k, v))
+        ks, vs = (t.repeat_interleave(n_heads // n_kv, 0) for t in (ks, vs))
+        score = (qs @ ks.transpose(1, 2) / math.sqrt(dh)).masked_fill(torch.ones(n, n, device="cuda").triu(1).bool(), -math.inf)
+        parts.append((score.softmax(-1) @ vs).transpose(0, 1).reshape(n, d))
+    x2 = x + lin("o", torch.cat(parts))
+    h2 = norm(x2, w["g2"])
+    return x2 + lin("down", torch.nn.functional.silu(lin("gate", h2)) * lin("up", h2))
+
+
+def exact(case, seed):
+    """What `run` returns on a state just prepared, from the definitions in 64 bits."""
+    c = dict(_DEFAULTS, **case)
+    s = prepare(case, seed)
+    b = _Mixed64(c, seed)
+    if c["kind"] != "layer":
+        return [b.projection(c, p) for p in s.projections.values()]
+    layer, w = s.layer, {"g1": s.layer.g1.double(), "g2": s.layer.g2.double()}
+    for name, p in layer.proj.items():
+        w["W_" + name], w["A_" + name], w["B_" + name], w["s_" + name] = p.W, p.A.double(), p.B.double(), p.scale
+    x = s.x.double()
+    with torch.no_grad():
+        y = _layer64(b, x, w, c["heads"], c["kv_heads"])
+    if not c["backward"]:
+        return [y]
+    f = b.first
+    leaf = x[f:].clone().requires_grad_(True)
+    wanted = [w[k + n].requires_grad_(True) for n in layer.proj for k in ("A_", "B_")]
+    with torch.enable_grad():
+        got = torch.autograd.grad(_layer64(b, leaf, w, c["heads"], c["kv_heads"], f), [leaf] + wanted, s.dy.double())
+    grads = {n: (got[1 + 2 * i][b.slots], got[2 + 2 * i][b.slots]) for i, n in enumerate(layer.proj)}
+    return [y, got[0], grads]
+
+
 # ---- the work of a case and how exact its results are ----------------------------------------------
 def _distinct(c):
     """Adapters that a batch meets, in the mean over seeds."""
