@@ -1,0 +1,393 @@
+// Few-row variant of the fused GEMM + LoRA-expand kernel (see gemm_tcgen05.cuh for the operator): decode steps and the
+// backward batches of one or two fine-tuning sequences.
+//
+// What bounds such a product is the one pass over the weight, so the operands change places: a 128-column block of
+// the weight is the M = 128 side of the MMA and the batch rows are its N side (16 to 128, padded to 16), and every
+// CTA holds a deep ring of weight blocks in flight.  The 256 x 256 tiles of the two-SM kernel give a 4096-wide
+// output 16 work units for 74 CTA pairs; here it has 32 column blocks, each cut along K over the CTAs of a cluster
+// (up to 8), which add their fp32 accumulators over distributed shared memory in slice order - no fp32 partials in
+// global memory and no second launch to add them.
+//
+// The kernel also hides the rank-r product in front of it: neither the weight nor the input rows come from the
+// launch before (the shrink, or in the backward the gradient kernel), so with `early` set the main loop starts while
+// that launch still runs and only the low-rank blocks, which are the last ones of every slice, wait for it.  The host
+// sets `early` only behind a kernel of this library that lets its dependents start after its own dependency wait:
+// everything older than that kernel has then completed.
+//
+// Warp roles (224 threads): warp 0 loads weight blocks, warp 6 input rows, warp 1 issues the MMAs (owns tensor
+// memory), warps 2-5 first look up the tile's low-rank tables, then write the result.  Every wait is bounded, and all
+// threads meet in the block and cluster barriers on every path.
+#pragma once
+
+#include <cuda.h>
+
+#include <type_traits>
+
+#include "gemm_tcgen05.cuh"
+#include "ptx.cuh"
+
+namespace mlora {
+namespace rows {
+
+constexpr int BM = 128;                              // output columns of a CTA's tile (UMMA M)
+constexpr int THREADS = 224;
+constexpr uint32_t W_BYTES = BM * GEMM_BK * 2;       // 16 KiB: one K-block of the weight
+constexpr int MAX_STAGES = 8;
+constexpr int MAX_BOXES = 2048;                      // 256 groups of a 256-row tile x 128 / 16 pieces
+
+struct Args {
+  int32_t M, N, K;              // batch rows, output columns, contraction
+  int32_t nb;                   // rows of a tile (the MMA's N): a multiple of 16, at most 128; no tile straddles a multiple of 256
+  int32_t col_tiles;
+  int32_t stages;               // ring depth
+  int32_t slices;               // CTAs of a cluster = K slices of a tile
+  int32_t R;                    // rank
+  int32_t lora;                 // 0: base product only
+  int32_t early;                // 1: weight and input rows may be read before the dependency wait
+  const __nv_bfloat16* L_all;   // stacked adapter matrices [adapters R, N]
+  const int32_t* tile_grp_off;  // groups of each 256-row tile of the batch, and their adapters
+  const int32_t* grp_adapter;
+  const int32_t* tile_cols;     // plans made with per-adapter ranks (else null): columns of a tile's low-rank operand, first
+  const int32_t* grp_col;          // column of each group,
+  const int32_t* tile_piece_off;   // and its B side as 16-row pieces of the adapters' matrices
+  const int32_t* piece_src;
+  __nv_bfloat16* Out;           // [M, N]
+  int64_t ld_out;
+  int32_t* status;
+};
+
+// A stage holds KW K-blocks of the weight and of the rows.
+__host__ __device__ __forceinline__ uint32_t stage_bytes(int nb, int kw) { return (uint32_t)kw * (W_BYTES + (uint32_t)nb * 128u); }
+// Rows of a tile that one of its slices finishes.
+__host__ __device__ __forceinline__ int slice_rows(int nb, int slices) { return (nb + slices - 1) / slices; }
+// Ring (afterwards two buffers of [row][128] floats: the sums that leave and the sums that arrive) and its alignment.
+__host__ __device__ __forceinline__ uint32_t smem_bytes(int nb, int kw, int stages, int slices) {
+  const uint32_t ring = stage_bytes(nb, kw) * (uint32_t)stages, sums = (uint32_t)(slice_rows(nb, slices) * slices) * 1024u;
+  return (ring > sums ? ring : sums) + 1024u;
+}
+
+// Place in the ring: slot and the parity of its current use.
+struct Ring {
+  int n, slot = 0;
+  uint32_t parity = 0;
+  __device__ explicit Ring(int stages) : n(stages) {}
+  __device__ __forceinline__ void next() { if (++slot == n) { slot = 0; parity ^= 1; } }
+};
+
+// Shared memory of this CTA -> shared memory of a CTA of the cluster, bytes counted on a barrier of that CTA.
+__device__ __forceinline__ void bulk_to_cta(uint32_t dst_cluster, uint32_t src, uint32_t bytes, uint32_t bar_cluster) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst_cluster), "r"(src), "r"(bytes), "r"(bar_cluster) : "memory");
+}
+
+// grid = row tiles x column tiles x slices, clusters of `slices` CTAs: cluster = output tile, rank in it = K slice.
+// KW = K-blocks per stage: two halve the barrier and issue cost per block where the rows leave room for a deep ring.
+template <bool W_KMAJOR, int KW>
+__global__ void __launch_bounds__(THREADS, 1)
+gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ CUtensorMap tmW,
+                 const __grid_constant__ CUtensorMap tmL, const __grid_constant__ CUtensorMap tmPbd, const Args args) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES + 2];      // full | empty | accumulator complete | peers' sums
+  __shared__ int32_t box_row[MAX_BOXES];                          // row in the stacked adapter matrices of each low-rank box
+  __shared__ int32_t lora_info[3];                                // this slice's columns of the tile's low-rank operand, its first group
+  __shared__ uint32_t tmem_ptr;
+  __shared__ int abort_word;
+  volatile int* abort_flag = &abort_word;
+  const uint32_t ring = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* ring_gen = smem_raw + (ring - ptx::smem_u32(smem_raw));
+  const uint32_t bar0 = ptx::smem_u32(bars);
+  auto bar_full = [&](int s) { return bar0 + 8u * s; };
+  auto bar_empty = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
+  const uint32_t bar_done = bar0 + 8u * (2 * MAX_STAGES), bar_sums = bar_done + 8u;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int S = args.stages, SK = args.slices, nb = args.nb;
+  const int tile = (int)blockIdx.x / SK, ks = (int)blockIdx.x - tile * SK;
+  const int rt = tile / args.col_tiles;
+  const int m0 = rt * nb, n0 = (tile - rt * args.col_tiles) * BM;
+  const int rows_here = args.M - m0 < nb ? args.M - m0 : nb;
+  const uint32_t xblk = (uint32_t)nb * 128u, stage = KW * (W_BYTES + xblk);
+  uint32_t tmem_cols = 32;
+  while (tmem_cols < (uint32_t)nb) tmem_cols *= 2;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      ptx::mbar_init(bar_full(s), 2);          // both producers
+      ptx::mbar_init(bar_empty(s), 1);
+    }
+    ptx::mbar_init(bar_done, 1);
+    ptx::mbar_init(bar_sums, 1);
+    abort_word = 0;
+    ptx::fence_barrier_init();
+    ptx::prefetch_tmap(&tmIn);
+    ptx::prefetch_tmap(&tmW);
+    ptx::prefetch_tmap(&tmL);
+    ptx::prefetch_tmap(&tmPbd);
+  }
+  if (warp == 1) {
+    ptx::tmem_alloc(ptx::smem_u32(&tmem_ptr), tmem_cols);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = tmem_ptr;
+  if (!args.early) ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();
+
+  const int KB = (args.K + KW * GEMM_BK - 1) / (KW * GEMM_BK);
+  const int kb_begin = (int)((long long)ks * KB / SK), kb_end = (int)((long long)(ks + 1) * KB / SK);
+  // The tile's low-rank tables are looked up by the epilogue warps while the main loop runs (named barriers 1, 3, 4: they
+  // arrive, the other roles each wait behind their main blocks).
+  // A slice takes whole adapter groups, the same ones however wide a plan packs them: columns [col_begin, col_end) of the
+  // operand, both multiples of 16 but for the end of an odd number of groups of rank 8.
+  int col_begin = 0, col_end = 0, grp0 = 0;
+  auto lora_range = [&]() { col_begin = lora_info[0]; col_end = lora_info[1]; grp0 = lora_info[2]; };
+  // A producer that gives up lets its loads in flight land (bounded: the other producer may not have filled the slot).
+  auto drain = [&](const Ring& at) {
+    for (uint32_t i = 0; i < (1u << 12) && !ptx::mbar_try_wait(bar_full(at.slot), at.parity); ++i) {}
+  };
+  const int box = args.piece_src ? 16 : (args.R < 64 ? args.R : 64);      // rows of an adapter's matrix per low-rank load
+  const int per = 64 / box;
+
+  if (warp == 0) {
+    // ============================ TMA producer: weight blocks, then the adapters' rows ============================
+    Ring at(S);
+    int ok = 1;
+    if (lane == 0) {
+      for (int kb = kb_begin; kb < kb_end; ++kb, at.next()) {
+        if (!(ok = gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status))) break;
+        const uint32_t w = ring + (uint32_t)at.slot * stage, full = bar_full(at.slot);
+        ptx::mbar_arrive_expect_tx(full, KW * W_BYTES);
+        if (W_KMAJOR) ptx::tma_load_3d(w, &tmW, 0, n0, kb * KW, full);                   // (64 k, N, K/64): KW blocks of 128 rows x 64 k
+        else          ptx::tma_load_3d(w, &tmW, 0, kb * KW * GEMM_BK, n0 >> 6, full);    // (64 n, K, N/64): 2 blocks of 64 KW k x 64 n
+      }
+    }
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+    at.slot = __shfl_sync(0xffffffffu, at.slot, 0);
+    at.parity = __shfl_sync(0xffffffffu, at.parity, 0);
+    asm volatile("bar.sync 1, 160;" ::: "memory");
+    lora_range();
+    const int box_begin = col_begin / box, box_end = (col_end + box - 1) / box;
+    for (int lc = col_begin / 64; lc * 64 < col_end && ok; lc += KW, at.next()) {
+      if (lane == 0) ok = gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      if (!ok) break;
+      const int j0 = box_begin > lc * per ? box_begin : lc * per, j1 = box_end < (lc + KW) * per ? box_end : (lc + KW) * per;
+      const int n = box == 8 ? (j1 - j0 + 1) & ~1 : j1 - j0;     // rank 8: a half-filled MMA step repeats the last group (its operand columns are zero)
+      const uint32_t w = ring + (uint32_t)at.slot * stage, full = bar_full(at.slot);
+      if (lane == 0) ptx::mbar_arrive_expect_tx(full, (uint32_t)(n * box) * 256u);
+      __syncwarp();
+      if (lane < n) {                      // one box per lane, both 64-column halves: [half][box rows][64]
+        const int j = j0 + lane;
+        ptx::tma_load_3d(w + (uint32_t)((j - lc * per) * box) * 256u, &tmL, 0, box_row[j < j1 ? j : j1 - 1], n0 >> 6, full);
+      }
+    }
+    if (!ok && lane == 0) drain(at);
+    __syncwarp();
+  } else if (warp == 6) {
+    // ============================ TMA producer: input rows, then their low-rank operand ============================
+    Ring at(S);
+    int ok = 1;
+    if (lane == 0) {
+      for (int kb = kb_begin; kb < kb_end; ++kb, at.next()) {
+        if (!(ok = gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status))) break;
+        const uint32_t x = ring + (uint32_t)at.slot * stage + KW * W_BYTES, full = bar_full(at.slot);
+        ptx::mbar_arrive_expect_tx(full, KW * xblk);
+        ptx::tma_load_3d(x, &tmIn, 0, m0, kb * KW, full);                          // (64 k, M, K/64): KW blocks of nb rows x 64 k
+      }
+    }
+    __syncwarp();
+    asm volatile("bar.sync 3, 160;" ::: "memory");
+    lora_range();
+    if (lane == 0) {
+      if (args.early && col_begin < col_end) ptx::grid_dependency_wait();            // the operand comes from the launch before
+      for (int lc = col_begin / 64; lc * 64 < col_end && ok; lc += KW, at.next()) {
+        if (!(ok = gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status))) break;
+        const uint32_t x = ring + (uint32_t)at.slot * stage + KW * W_BYTES, full = bar_full(at.slot);
+        const int n = KW == 1 || (lc + 1) * 64 >= col_end ? 1 : KW;
+        ptx::mbar_arrive_expect_tx(full, (uint32_t)n * xblk);
+        for (int b = 0; b < n; ++b)
+          ptx::tma_load_2d(x + (uint32_t)b * xblk, &tmPbd, 0, (2 * grp0 + lc + b) * 256 + (m0 & 255), full);
+      }
+      if (!ok) drain(at);
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ============================ MMA issuer ============================
+    // Both loops are unrolled with constant descriptor offsets: with a runtime trip count every MMA waited for its
+    // operands to reach the uniform registers (790 clocks per K-block whatever its width).
+    const uint32_t idesc_main = ptx::make_idesc_bf16(BM, (uint32_t)nb, !W_KMAJOR, false);
+    const uint32_t idesc_lora = ptx::make_idesc_bf16(BM, (uint32_t)nb, true, false);
+    uint32_t acc = 0;
+    int ok = 1;
+    Ring at(S);
+    if (lane == 0) {
+      for (int kb = kb_begin; kb < kb_end; ++kb, at.next()) {
+        if (!(ok = gemm_wait(bar_full(at.slot), at.parity, abort_flag, args.status))) break;
+        ptx::tc_fence_after();
+        const uint32_t w = ring + (uint32_t)at.slot * stage;
+        const uint64_t adesc = W_KMAJOR ? ptx::make_smem_desc(w, 16, 1024) : ptx::make_smem_desc(w, KW * 8192, 1024);
+        const uint64_t bdesc = ptx::make_smem_desc(w + KW * W_BYTES, 16, 1024);
+#pragma unroll
+        for (int b = 0; b < KW; ++b)
+#pragma unroll
+          for (int k = 0; k < GEMM_BK / 16; ++k) {
+            ptx::umma_f16(tmem_base, adesc + (uint64_t)(W_KMAJOR ? b * (W_BYTES >> 4) + k * 2 : (b * 4 + k) * 128),
+                          bdesc + (uint64_t)(b * (xblk >> 4) + k * 2), idesc_main, acc);
+            acc = 1;
+          }
+        ptx::umma_commit(bar_empty(at.slot));
+      }
+    }
+    __syncwarp();
+    asm volatile("bar.sync 4, 160;" ::: "memory");
+    lora_range();
+    if (lane == 0) {
+      // boxes of [2 halves][BOX rows][64 columns]: 16 operand columns are 16 rows of one box, or two boxes of 8
+      auto lora_mma = [&](auto box_rows) {
+        constexpr int BOX = decltype(box_rows)::value;
+        for (int lc = col_begin / 64; lc * 64 < col_end && ok; lc += KW, at.next()) {
+          if (!(ok = gemm_wait(bar_full(at.slot), at.parity, abort_flag, args.status))) break;
+          ptx::tc_fence_after();
+          const uint32_t w = ring + (uint32_t)at.slot * stage;
+          const uint64_t adesc = ptx::make_smem_desc(w, BOX * 128, BOX == 8 ? 2048 : 1024);
+          const uint64_t bdesc = ptx::make_smem_desc(w + KW * W_BYTES, 16, 1024);
+          const int from = col_begin - lc * 64, to = col_end - lc * 64;
+#pragma unroll
+          for (int k = 0; k < KW * (GEMM_BK / 16); ++k)
+            if (k * 16 >= from && k * 16 < to) {
+              constexpr int per_box = BOX < 16 ? 1 : BOX / 16;
+              const uint32_t at_k = BOX == 8 ? k * 4096 : (k / per_box) * BOX * 256 + (k % per_box) * 2048;
+              ptx::umma_f16(tmem_base, adesc + (uint64_t)(at_k >> 4),
+                            bdesc + (uint64_t)((k >> 2) * (xblk >> 4) + (k & 3) * 2), idesc_lora, acc);
+              acc = 1;
+            }
+          ptx::umma_commit(bar_empty(at.slot));
+        }
+      };
+      if (box == 8) lora_mma(std::integral_constant<int, 8>());
+      else if (box == 16) lora_mma(std::integral_constant<int, 16>());
+      else if (box == 32) lora_mma(std::integral_constant<int, 32>());
+      else lora_mma(std::integral_constant<int, 64>());
+      if (ok) ptx::umma_commit(bar_done);
+    }
+    __syncwarp();
+  } else {
+    // ============================ low-rank tables (plan data: not written by any kernel) ============================
+    const int t = (int)threadIdx.x - 64, mt = m0 >> 8;
+    const int g = args.lora ? args.tile_grp_off[mt] : 0;
+    const int n_grp = args.lora ? args.tile_grp_off[mt + 1] - g : 0;
+    if (args.piece_src) {
+      const int p = args.tile_piece_off[mt], n = args.lora ? args.tile_piece_off[mt + 1] - p : 0;
+      for (int j = t; j < n && j < MAX_BOXES; j += 128) {
+        const int src = args.piece_src[p + j];
+        box_row[j] = (src >> 8) * args.R + (src & 255) * 16;
+      }
+    } else {
+      const int per_grp = args.R > 64 ? args.R / 64 : 1;
+      for (int j = t; j < n_grp * per_grp && j < MAX_BOXES; j += 128)
+        box_row[j] = args.grp_adapter[g + j / per_grp] * args.R + (j % per_grp) * 64;
+    }
+    if (t < 2) {                                             // first column of this slice's first group, and of the next slice's
+      int gi = (int)((long long)(ks + t) * n_grp / SK);
+      if (args.R == 8 && ks + t < SK) gi &= ~1;
+      lora_info[t] = !args.tile_cols ? gi * args.R : (gi < n_grp ? args.grp_col[g + gi] : (args.lora ? args.tile_cols[mt] : 0));
+    }
+    if (t == 2) lora_info[2] = g;
+    asm volatile("bar.sync 2, 128;" ::: "memory");
+    asm volatile("bar.arrive 1, 160;\n\tbar.arrive 3, 160;\n\tbar.arrive 4, 160;" ::: "memory");
+    lora_range();
+    // The adapters' rows of this tile are 128-byte pieces all over memory: on their way to the L2 while the main blocks
+    // stream, so that the low-rank blocks behind them do not wait for memory one after the other.
+    for (int i = col_begin + t; i < col_end; i += 128) {
+      const __nv_bfloat16* p = args.L_all + (size_t)(box_row[i / box] + i % box) * args.N + n0;
+      ptx::prefetch_l2(p);
+      if (n0 + 64 < args.N) ptx::prefetch_l2(p + 64);
+    }
+    gemm_wait(bar_done, 0, abort_flag, args.status);
+    ptx::tc_fence_after();
+    // no CTA ends before the launch ahead of it has: what follows in the stream may rely on that
+    ptx::grid_dependency_wait();
+  }
+  __syncwarp();
+
+  // ============================ the slices' sums ============================
+  // Every CTA is done with its ring (its own MMAs have completed, or it gave up and drained its loads), so the rings
+  // take the fp32 sums: slice d of the cluster finishes rows [d chunk, (d + 1) chunk) of all 128 columns.  Each CTA lays
+  // its accumulator out as [row][128] and sends every peer its rows as one bulk copy (scalar stores to the peers moved
+  // 10 bytes a clock); the sums that arrive land as [slice][row][128] behind them and are added in slice order.
+  __syncthreads();
+  if (SK > 1) ptx::cluster_sync_all();
+  if (warp >= 2 && warp < 6) {
+    const int chunk = slice_rows(nb, SK);
+    const uint32_t part = (uint32_t)chunk * (BM * 4u);              // bytes of one slice's share
+    const uint32_t arrived = ring + (uint32_t)SK * part;
+    const int e = warp & 3;
+    const uint32_t taddr = tmem_base + ((uint32_t)(e * 32) << 16);
+    const uint32_t mine = ring + (uint32_t)(e * 32 + lane) * 4u;
+    for (int j0 = 0; j0 < rows_here; j0 += 16) {
+      uint32_t v[16];
+      ptx::tmem_ld_32x32b_x16(taddr + j0, v);
+      ptx::tmem_ld_wait();
+#pragma unroll
+      for (int j = 0; j < 16; ++j) asm volatile("st.shared.b32 [%0], %1;" ::"r"(mine + (uint32_t)(j0 + j) * (BM * 4u)), "r"(v[j]) : "memory");
+    }
+    ptx::fence_proxy_async_smem();
+    ptx::tc_fence_before();
+    asm volatile("bar.sync 2, 128;" ::: "memory");
+    if (SK > 1) {
+      if (threadIdx.x == 64) {
+        ptx::mbar_arrive_expect_tx(bar_sums, (uint32_t)(SK - 1) * part);
+        for (int i = 1; i < SK; ++i) {
+          const int d = (ks + i) % SK;
+          bulk_to_cta(ptx::map_to_cta(arrived + (uint32_t)ks * part, (uint32_t)d), ring + (uint32_t)d * part, part,
+                      ptx::map_to_cta(bar_sums, (uint32_t)d));
+        }
+      }
+      gemm_wait(bar_sums, 0, abort_flag, args.status);
+    }
+    // 16 threads per row, eight columns each
+    const int t = (int)threadIdx.x - 64, c8 = (t & 15) * 8;
+    const int r_end = rows_here - ks * chunk < chunk ? rows_here - ks * chunk : chunk;
+    if (n0 + c8 < args.N && *abort_flag == 0) {
+      __nv_bfloat16* out = args.Out + (size_t)(m0 + ks * chunk) * args.ld_out + n0 + c8;
+      const uint8_t* own = ring_gen + (size_t)ks * part;
+      const uint8_t* others = ring_gen + (size_t)SK * part;
+      for (int r0 = t >> 4; r0 < r_end; r0 += 32) {                  // four rows in flight
+        float sum[4][8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) sum[i][j] = 0.f;
+        for (int s = 0; s < SK; ++s) {
+          const uint8_t* from = (s == ks ? own : others + (size_t)s * part) + (size_t)(r0 * BM + c8) * 4;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            if (r0 + 8 * i >= r_end) break;
+            const float4* src = reinterpret_cast<const float4*>(from + (size_t)(8 * i * BM) * 4);
+            const float4 a = src[0], b = src[1];
+            sum[i][0] += a.x; sum[i][1] += a.y; sum[i][2] += a.z; sum[i][3] += a.w;
+            sum[i][4] += b.x; sum[i][5] += b.y; sum[i][6] += b.z; sum[i][7] += b.w;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (r0 + 8 * i < r_end)
+            *reinterpret_cast<uint4*>(out + (size_t)(r0 + 8 * i) * args.ld_out) =
+                make_uint4(ptx::pack_bf16(sum[i][0], sum[i][1]), ptx::pack_bf16(sum[i][2], sum[i][3]),
+                           ptx::pack_bf16(sum[i][4], sum[i][5]), ptx::pack_bf16(sum[i][6], sum[i][7]));
+      }
+    }
+  }
+  __syncwarp();
+  __syncthreads();
+  if (SK > 1) ptx::cluster_sync_all();       // the copies out of this CTA's memory have arrived at their peers
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem_base, tmem_cols);
+  }
+}
+
+}  // namespace rows
+}  // namespace mlora

@@ -19,6 +19,7 @@
 #include "plan.h"
 #include "gemm_tcgen05.cuh"
 #include "gemm2_tcgen05.cuh"
+#include "gemm_rows_tcgen05.cuh"
 #include "simt.cuh"
 #include "skinny.cuh"
 #include "grad_tc.cuh"
@@ -302,17 +303,17 @@ void launch_pdl(bool overlap, void (*kern)(KArgs...), dim3 grid, dim3 block, siz
   cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-// Same, for a kernel whose CTAs come in clusters of two.
+// Same, for a kernel whose CTAs come in clusters.
 template <typename... KArgs, typename... Args>
-void launch_pdl_pairs(bool overlap, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                      Args&&... args) {
+void launch_pdl_cluster(bool overlap, void (*kern)(KArgs...), dim3 grid, dim3 block, dim3 cluster, size_t smem, cudaStream_t st,
+                        Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
   at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = 2; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  at[1].val.clusterDim.x = cluster.x; at[1].val.clusterDim.y = cluster.y; at[1].val.clusterDim.z = cluster.z;
   cfg.attrs = at; cfg.numAttrs = 2;
   cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
@@ -323,6 +324,94 @@ void launch_shrink_rb(bool overlap, const ShrinkArgs& a, int n_items, int ksplit
   launch_pdl(overlap, shrink_kernel<RB, MT, WARPS, MIN_CTAS>, dim3(n_items, ksplit, kItemRows / (16 * MT)),
              dim3(WARPS * 32), 0, st, a);
 }
+// Resident clusters of 1 to 8 CTAs of the few-row GEMM (nullptr: the query failed).  Its ring takes more than half of an
+// SM's shared memory, so that no two of its CTAs ever share an SM (their tensor memory might not fit beside a neighbour's
+// while each waits for the rest of its cluster), and little enough that CTAs of the shrink in front of it do.
+constexpr int kRowsRing = 144 << 10;
+const int* rows_clusters(const mlora_ctx* ctx) {
+  static int clusters_dev[kMaxDevices][9] = {};
+  int* clusters = clusters_dev[ctx->device];
+  std::lock_guard<std::mutex> lock(g_attr_mutex);
+  if (clusters[1] > 0) return clusters;
+  const size_t smem = kRowsRing + 1024;
+  if (cudaFuncSetAttribute(rows::gemm_rows_kernel<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaFuncSetAttribute(rows::gemm_rows_kernel<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaFuncSetAttribute(rows::gemm_rows_kernel<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaFuncSetAttribute(rows::gemm_rows_kernel<true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  for (int c = 8; c >= 1; --c) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctx->sm_count / c * c); cfg.blockDim = dim3(rows::THREADS); cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = c; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, rows::gemm_rows_kernel<false, 1>, &cfg) != cudaSuccess || n <= 0) { cudaGetLastError(); return nullptr; }
+    clusters[c] = n;
+  }
+  return clusters;
+}
+
+// Rows of a tile, K-blocks per stage and K slices of the few-row GEMM for an [M, K] x [K, N] product, or false: the two-SM
+// kernel's product.  Measured on B200 (whole forward calls, 4 adapters of rank 16, two-SM path / this one, us):
+//   4096 -> 4096:   16 rows 21.3 / 12.8, 64 24.3 / 14.2, 128 27.2 / 16.2, 256 28.2 / 20.9, 512 35.7 / 29.1
+//   4096 -> 14336:  16 rows 34.1 / 24.0, 128 36.4 / 30.8, but 192 36.9 / 54.6 and 512 63.8 / 119 (224 and more tiles: two
+//                   rounds of CTAs), hence at most one tile per SM
+//   10880 -> 2816:  64 rows 33.1 / 21.0, 256 37.1 / 29.4 (57 K-blocks per slice), but 512 46.7 / 62.7 (170 per slice)
+//   12288-deep input gradient: 192 rows 54.5 / 60.0 (96 per slice), hence at most 64 K-blocks per slice where the rows of a
+//   tile are many enough (above 64) for the L2 traffic of a block to be what it costs (0.34 us at 128 rows).
+// Slices: as many as clusters of that size are resident at once, with at least 8 K-blocks each.  Clusters of 3, 5 and 7
+// straddle SM pairs and do not all find room while the launch in front still holds SMs (44 of 45 clusters of 3: 28 us in a
+// row of launches of its own kind, 39 behind the streaming shrink), so those count for nine tenths.
+struct RowsShape { int nb, kw, slices; };
+bool rows_shape(const mlora_ctx* ctx, int M, int N, int K, RowsShape& r) {
+  if (ctx->gemm_path != 0 || ctx->shrink_path != 0 || !ctx->gemm_pairs || ctx->no_split_k || ctx->grad_mode != 0) return false;
+  r.nb = M <= 128 ? (M + 15) / 16 * 16 : (M <= 256 ? ((M + 1) / 2 + 15) / 16 * 16 : 128);
+  const int64_t tiles = (int64_t)((N + rows::BM - 1) / rows::BM) * ((M + r.nb - 1) / r.nb);
+  if (tiles > ctx->sm_count) return false;
+  const int* clusters = rows_clusters(ctx);
+  if (!clusters) return false;
+  const int kblocks = K / GEMM_BK;
+  r.slices = 1;
+  for (int c = 2; c <= 8; ++c)
+    if (kblocks / c >= 8 && tiles <= ((c & 1) ? clusters[c] * 9 / 10 : clusters[c])) r.slices = c;
+  r.kw = r.nb <= 64 ? 2 : 1;
+  return r.nb <= 64 || kblocks / r.slices <= 64;
+}
+
+// Shrink of a batch of few rows: items x a cluster along K, as many CTAs as two per SM.
+template <int R, int MT, bool DROP>
+mlora_status_t launch_shrink_few_d(mlora_ctx* ctx, const ShrinkArgs& a, int n_items, cudaStream_t st) {
+  static bool attr_set_dev[kMaxDevices] = {};   // per instantiation and device
+  auto kern = shrink_few_kernel<R, MT, DROP>;
+  {
+    // The GEMM behind this kernel moves onto the same SMs only if their shared memory is already carved out in full.
+    std::lock_guard<std::mutex> lock(g_attr_mutex);
+    if (!attr_set_dev[ctx->device]) {
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess) return MLORA_ERR_CUDA;
+      attr_set_dev[ctx->device] = true;
+    }
+  }
+  const int parts = R > 32 ? R / 32 : 1, z = parts * (kItemRows / (16 * MT)), nkb = a.D / 64;
+  int cl = 1;
+  while (cl < 8 && cl * n_items * parts <= ctx->sm_count && nkb >= 2 * cl * FEW_WARPS) cl *= 2;
+  if (cancelled(ctx)) return MLORA_CANCELLED;
+  LaunchScope scope(ctx, st, KIND_SHRINK);
+  launch_pdl_cluster(scope.slot < 0, kern, dim3(n_items, cl, z), dim3(FEW_WARPS * 32), dim3(1, cl, 1), 0, st, a);
+  return scope.done();
+}
+template <int R>
+mlora_status_t launch_shrink_few(mlora_ctx* ctx, ShrinkArgs a, int n_items, cudaStream_t st) {
+  if (a.item_save && ctx->drop.thr != 0) {      // only the forward's fine-tuning rows are dropped; the mask's arithmetic over twice the CTAs
+    a.drop = ctx->drop;
+    return launch_shrink_few_d<R, 1, true>(ctx, a, n_items, st);
+  }
+  return launch_shrink_few_d<R, (R < 32 ? 2 : 1), false>(ctx, a, n_items, st);
+}
+
 // Few items with a long contraction leave most SMs idle: split K over several CTAs per item so
 // that about three CTAs per SM are in flight, keeping at least 16 K-blocks (1024 elements) each.
 int shrink_ksplit(const mlora_ctx* ctx, int n_items, int D) {
@@ -395,8 +484,18 @@ mlora_status_t launch_shrink_stream(mlora_ctx* ctx, ShrinkArgs a, int n_items, c
 }
 
 mlora_status_t launch_shrink(mlora_ctx* ctx, int R, ShrinkArgs a, int n_items, const int32_t* item_desc, int n_rows,
-                             int n_adapters, cudaStream_t st) {
+                             int n_adapters, bool few, cudaStream_t st) {
   if (n_items <= 0) return MLORA_OK;
+  if (few) {
+    switch (R) {
+      case 8: return launch_shrink_few<8>(ctx, a, n_items, st);
+      case 16: return launch_shrink_few<16>(ctx, a, n_items, st);
+      case 32: return launch_shrink_few<32>(ctx, a, n_items, st);
+      case 64: return launch_shrink_few<64>(ctx, a, n_items, st);
+      case 128: return launch_shrink_few<128>(ctx, a, n_items, st);
+      default: return MLORA_ERR_UNSUPPORTED;
+    }
+  }
   if (ctx->shrink_path == 0) {
     if (R == 8) return launch_shrink_stream<1, 2, 16>(ctx, a, n_items, item_desc, n_rows, n_adapters, st);
     if (R == 16) return launch_shrink_stream<2, 2, 16>(ctx, a, n_items, item_desc, n_rows, n_adapters, st);
@@ -743,7 +842,7 @@ mlora_status_t launch_gemm2_r(mlora_ctx* ctx, const CUtensorMap& tIn, const CUte
   GemmArgs ga = g;
   if (ga.unit_list && ga.sched_pairs != pairs) ga.unit_list = nullptr;   // the list was made for another grid
   LaunchScope scope(ctx, st, W_KMAJOR ? KIND_GEMM_BWD : KIND_GEMM_FWD);
-  launch_pdl_pairs(scope.slot < 0, kern, dim3(2 * pairs), dim3(GEMM2_THREADS), GEMM2_SMEM_BYTES, st, tIn, tW, tL, tOut, tPbd, ga);
+  launch_pdl_cluster(scope.slot < 0, kern, dim3(2 * pairs), dim3(GEMM2_THREADS), dim3(2, 1, 1), GEMM2_SMEM_BYTES, st, tIn, tW, tL, tOut, tPbd, ga);
   return scope.done();
 }
 
@@ -881,11 +980,55 @@ inline void set_ranked(PbdArgs& pa, const DevRowSpace& ds) {
   pa.grp2_col = ds.grp2_col; pa.grp2_width = ds.grp2_width; pa.tile2_cols = ds.tile2_cols;
 }
 
-// Out = In Wop + (scale) P L over one row space, tensor-core path.
+// The few-row kernel: one cluster per (row tile, column tile), its CTAs the K slices.
+template <bool W_KMAJOR, int KW>
+mlora_status_t launch_gemm_rows(mlora_ctx* ctx, const mlora_layer_t* L, const RowSpace& hs, const DevRowSpace& ds, const void* In,
+                                int64_t ld_in, void* Out, int64_t ld_out, const void* L_all, int M, int N, int K, const RowsShape& shape,
+                                bool lora, bool early, cudaStream_t st) {
+  const int R = L->rank, nb = shape.nb;
+  const bool ranked = ds.piece_src != nullptr;
+  rows::Args a;
+  a.M = M; a.N = N; a.K = K; a.R = R; a.nb = nb;
+  a.lora = lora && !hs.grp2_adapter.empty() ? 1 : 0;
+  a.early = early ? 1 : 0;
+  a.L_all = (const __nv_bfloat16*)L_all;
+  a.tile_grp_off = ds.tile2_grp_off; a.grp_adapter = ds.grp2_adapter;
+  a.tile_cols = ranked ? ds.tile2_cols : nullptr; a.grp_col = ds.grp2_col; a.tile_piece_off = ds.tile2_piece_off; a.piece_src = ranked ? ds.piece_src : nullptr;
+  a.Out = (__nv_bfloat16*)Out; a.ld_out = ld_out; a.status = ctx->status_dev;
+  a.col_tiles = (N + rows::BM - 1) / rows::BM;
+  const int tiles = a.col_tiles * ((M + nb - 1) / nb);
+  a.slices = shape.slices;
+  a.stages = kRowsRing / (int)rows::stage_bytes(nb, KW);
+  a.stages = a.stages < rows::MAX_STAGES ? a.stages : rows::MAX_STAGES;
+  CUtensorMap tIn, tW, tL, tPbd;
+  mlora_status_t s;
+  if ((s = make_tmap_bf16_blocked(ctx, &tIn, In, M, K, ld_in, nb, KW)) != MLORA_OK) return s;
+  if (W_KMAJOR) s = make_tmap_bf16_blocked(ctx, &tW, L->W, N, K, L->ldw, rows::BM, KW);
+  else          s = make_tmap_bf16_blocked(ctx, &tW, L->W, K, N, L->ldw, KW * GEMM_BK, 2);
+  if (s != MLORA_OK) return s;
+  tL = tW; tPbd = tIn;
+  if (a.lora) {
+    if ((s = make_tmap_bf16_blocked(ctx, &tL, L_all, (uint64_t)L->n_adapters * R, N, N, ranked ? 16 : (R < 64 ? R : 64), 2)) != MLORA_OK) return s;
+    if ((s = make_tmap_bf16(ctx, &tPbd, ctx->ws_pbd, 64, (uint64_t)hs.grp2_adapter.size() * 512, 64, 64, nb)) != MLORA_OK) return s;
+  }
+  if (cancelled(ctx)) return MLORA_CANCELLED;
+  LaunchScope scope(ctx, st, W_KMAJOR ? KIND_GEMM_BWD : KIND_GEMM_FWD);
+  launch_pdl_cluster(scope.slot < 0, rows::gemm_rows_kernel<W_KMAJOR, KW>, dim3(tiles * a.slices), dim3(rows::THREADS), dim3(a.slices, 1, 1),
+                     rows::smem_bytes(nb, KW, a.stages, a.slices), st, tIn, tW, tL, tPbd, a);
+  return scope.done();
+}
+
+// Out = In Wop + (scale) P L over one row space, tensor-core path.  `early`: the launch in front of this one in the stream
+// is this call's own rank-r or gradient kernel (see gemm_rows_tcgen05.cuh).
 template <bool W_KMAJOR>
 mlora_status_t gemm_bf16(mlora_ctx* ctx, const mlora_layer_t* L, const RowSpace& hs, const DevRowSpace& ds,
                          const void* In, int64_t ld_in, void* Out, int64_t ld_out, const void* L_all,
-                         const float* P, const float* scale, int M, int N, int K, cudaStream_t st, bool lora = true) {
+                         const float* P, const float* scale, int M, int N, int K, cudaStream_t st, bool early, bool lora = true) {
+  RowsShape shape;
+  if (rows_shape(ctx, M, N, K, shape)) {
+    auto launch = shape.kw == 2 ? launch_gemm_rows<W_KMAJOR, 2> : launch_gemm_rows<W_KMAJOR, 1>;
+    return launch(ctx, L, hs, ds, In, ld_in, Out, ld_out, L_all, M, N, K, shape, lora, early, st);
+  }
   CUtensorMap tIn, tW, tL, tOut;
   mlora_status_t s;
   if ((s = make_tmap_bf16(ctx, &tIn, In, K, M, ld_in, GEMM_BK, GEMM_BM)) != MLORA_OK) return s;
@@ -1543,7 +1686,11 @@ mlora_status_t mlora_mixed_forward(mlora_ctx* ctx, const mlora_layer_t* L, const
   sa.x_save = (__nv_bfloat16*)x_save; sa.u_save = u_save; sa.save_base = save_row_base;
   sa.save_cap = save_capacity_rows;
   // rank >= kTcShrinkMinRank (every rank under kernel variant 6): the tcgen05 shrink and its finish kernel
-  const bool tc_shrink = ctx->shrink_path == 0 && ctx->drop.thr == 0 && !h.fwd.tcb_row0.empty() &&
+  // (a batch of few rows: the latency-bound shrink that its GEMM overlaps with; 10880 -> 2816, 128 rows: 28.4 -> 22.6 us
+  // for the whole call.  At ranks 64 and 128 the tcgen05 shrink is the faster one from 256 rows on, with or without overlap.)
+  RowsShape shape;
+  const bool few = h.n_rows <= (L->rank <= 32 ? 512 : 256) && rows_shape(ctx, h.n_rows, L->d_out, L->d_in, shape);
+  const bool tc_shrink = !few && ctx->shrink_path == 0 && ctx->drop.thr == 0 && !h.fwd.tcb_row0.empty() &&
                          (L->rank >= kTcShrinkMinRank || ctx->grad_mode == 2) && shrink_tc_fits(ctx, h.fwd, h.n_rows, L->d_in, L->rank);
   if (tc_shrink) {
     stc::FinArgs fa = {};
@@ -1552,11 +1699,11 @@ mlora_status_t mlora_mixed_forward(mlora_ctx* ctx, const mlora_layer_t* L, const
     fa.X = (const __nv_bfloat16*)X; fa.ldx = ldx; fa.x_save = (__nv_bfloat16*)x_save; fa.save_base = save_row_base; fa.D = L->d_in;
     s = launch_shrink_tc_any(ctx, L->rank, h.fwd, p->fwd, X, ldx, h.n_rows, L->d_in, L->A_all, L->n_adapters, fa, st);
   } else {
-    s = launch_shrink(ctx, L->rank, sa, h.fwd.n_items(), p->fwd.item_desc, h.n_rows, L->n_adapters, st);
+    s = launch_shrink(ctx, L->rank, sa, h.fwd.n_items(), p->fwd.item_desc, h.n_rows, L->n_adapters, few, st);
   }
   if (s != MLORA_OK) return s;
   return gemm_bf16<false>(ctx, L, h.fwd, p->fwd, X, ldx, Y, ldy, L->B_all, ctx->ws_p, L->scale, h.n_rows, L->d_out,
-                          L->d_in, st);
+                          L->d_in, st, h.fwd.n_items() > 0);
 }
 
 mlora_status_t mlora_backward(mlora_ctx* ctx, const mlora_layer_t* L, const mlora_plan* p, const void* dY, int64_t lddy,
@@ -1594,14 +1741,19 @@ mlora_status_t mlora_backward(mlora_ctx* ctx, const mlora_layer_t* L, const mlor
   set_ranked(sa.pbd, p->bwd);
   sa.item_adapter = p->bwd.item_adapter; sa.item_save = nullptr; sa.x_save = nullptr; sa.u_save = nullptr; sa.save_base = 0; sa.save_cap = 0;
   // V on the tcgen05 shrink from rank kTcShrinkMinRank (every rank under kernel variant 6), else on the mma.sync kernels
-  const bool tc_v = ctx->shrink_path == 0 && (L->rank >= kTcShrinkMinRank || ctx->grad_mode == 2) &&
+  // (few rows and a contraction short enough for the few-row kernel's four warps per slice: nothing overlaps with it here.
+  // Whole backward calls with it / with the others, us: 4096 -> 4096 rank 16, 64 rows 27.0 / 28.5; 2560 -> 3968 rank 128,
+  // 128 rows 38.6 / 39.9; 2816 -> 10880 rank 16, 64 rows 38.5 / 36.6; 2560 -> 3968 rank 128, 320 rows 53.0 / 49.9)
+  RowsShape shape;
+  const bool few = h.ft_rows <= 256 && L->d_out <= 6144 && rows_shape(ctx, h.ft_rows, L->d_in, L->d_out, shape);
+  const bool tc_v = !few && ctx->shrink_path == 0 && (L->rank >= kTcShrinkMinRank || ctx->grad_mode == 2) &&
                     shrink_tc_fits(ctx, h.bwd, h.ft_rows, L->d_out, L->rank);
   if (tc_v) {
     stc::FinArgs fa = {};
     fa.scale = L->scale; fa.Out = ctx->ws_p; fa.pbd = sa.pbd;
     s = launch_shrink_tc_any(ctx, L->rank, h.bwd, p->bwd, dY, lddy, h.ft_rows, L->d_out, L->B_all, L->n_adapters, fa, st);
   } else {
-    s = launch_shrink(ctx, L->rank, sa, h.bwd.n_items(), p->bwd.item_desc, h.ft_rows, L->n_adapters, st);
+    s = launch_shrink(ctx, L->rank, sa, h.bwd.n_items(), p->bwd.item_desc, h.ft_rows, L->n_adapters, few, st);
   }
   if (s != MLORA_OK) return s;
 
@@ -1632,7 +1784,7 @@ mlora_status_t mlora_backward(mlora_ctx* ctx, const mlora_layer_t* L, const mlor
     }
     if (s != MLORA_OK || !dX) return s;
     return gemm_bf16<true>(ctx, L, h.bwd, p->bwd, dY, lddy, dX, lddx, L->A_all, ctx->ws_p, nullptr, h.ft_rows, L->d_in,
-                           L->d_out, st);
+                           L->d_out, st, true);
   }
   if (ctx->shrink_path == 0 && L->rank <= 64) {      // both gradients in one launch of the streaming kernel
     s = L->rank <= 16 ? launch_grad_stream2<1>(ctx, p, ga, gA, n_slots, h.ft_rows, st)
@@ -1642,12 +1794,12 @@ mlora_status_t mlora_backward(mlora_ctx* ctx, const mlora_layer_t* L, const mlor
     if (!dX) return MLORA_OK;
     if (dropping) {   // the mask acts on the low-rank term per element: base product first, then the masked expand
       if ((s = gemm_bf16<true>(ctx, L, h.bwd, p->bwd, dY, lddy, dX, lddx, L->A_all, ctx->ws_p, nullptr, h.ft_rows,
-                               L->d_in, L->d_out, st, false)) != MLORA_OK)
+                               L->d_in, L->d_out, st, true, false)) != MLORA_OK)
         return s;
       return launch_expand_mask(ctx, L, p->bwd, dX, lddx, h.ft_rows, st);
     }
     return gemm_bf16<true>(ctx, L, h.bwd, p->bwd, dY, lddy, dX, lddx, L->A_all, ctx->ws_p, nullptr, h.ft_rows, L->d_in,
-                           L->d_out, st);
+                           L->d_out, st, true);
   }
   if ((s = launch_grad(ctx, p, ga, n_slots, h.ft_rows, st)) != MLORA_OK) return s;
   ga.P = ctx->ws_p; ga.scale = nullptr; ga.Q = (const __nv_bfloat16*)x_save; ga.ldq = L->d_in; ga.D = L->d_in;
@@ -1657,12 +1809,12 @@ mlora_status_t mlora_backward(mlora_ctx* ctx, const mlora_layer_t* L, const mlor
   if (!dX) return MLORA_OK;
   if (dropping) {   // the mask acts on the low-rank term per element: base product first, then the masked expand
     if ((s = gemm_bf16<true>(ctx, L, h.bwd, p->bwd, dY, lddy, dX, lddx, L->A_all, ctx->ws_p, nullptr, h.ft_rows, L->d_in,
-                             L->d_out, st, false)) != MLORA_OK)
+                             L->d_out, st, true, false)) != MLORA_OK)
       return s;
     return launch_expand_mask(ctx, L, p->bwd, dX, lddx, h.ft_rows, st);
   }
   return gemm_bf16<true>(ctx, L, h.bwd, p->bwd, dY, lddy, dX, lddx, L->A_all, ctx->ws_p, nullptr, h.ft_rows, L->d_in,
-                         L->d_out, st);
+                         L->d_out, st, true);
 }
 
 mlora_status_t mlora_adamw_update(mlora_ctx* ctx, const mlora_layer_t* L, const mlora_plan* p, const float* dA,

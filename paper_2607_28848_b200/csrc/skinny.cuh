@@ -271,6 +271,205 @@ shrink_kernel(const ShrinkArgs a) {
 }
 
 // ---------------------------------------------------------------------------------------------
+// Shrink of a batch of few rows (the few-row GEMM behind it, see gemm_rows_tcgen05.cuh).  Such a batch moves a few
+// megabytes at most, so the time is the chain of latencies: tables -> operands -> sum over the K split -> operand chunks
+// of the GEMM.  The K range of an item is split over a cluster of up to eight CTAs of four warps, the adapter's rows are
+// on their way to the L2 before the launch ahead has ended (a hint only: they are read behind the dependency wait), and
+// the cluster adds its parts over distributed shared memory in a fixed order - no partials in global memory, no counter,
+// no last arrival.  Ranks above 32 are cut into parts of 32 (a warp would otherwise wait for its adapter rows in four
+// rounds).  Small CTAs leave the GEMM room to start on the same SMs.
+// grid = (items, cluster, (R / 32 parts) x 32 / (16 MT)), clusters (1, cluster, 1); MT = 16-row blocks per CTA.
+constexpr int FEW_WARPS = 4;
+
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+template <int R, int MT, bool DROP>
+__global__ void __launch_bounds__(FEW_WARPS * 32, 4)
+shrink_few_kernel(const ShrinkArgs a) {
+  constexpr int RP = R < 32 ? R : 32, RB = RP / 8;          // ranks of this CTA's part, in column blocks of 8
+  constexpr int PARTS = R / RP;
+  constexpr int PITCH = RP + 2;                             // float2 accesses stay aligned
+  __shared__ __align__(16) float sum[MT * 16][PITCH];
+  __shared__ __align__(16) float fin[FEW_WARPS][RP];
+
+  const int part = blockIdx.z % PARTS, q_base = part * RP;
+  const int roff = blockIdx.z / PARTS * MT * 16;
+  const int nrows_item = a.item_nrows[blockIdx.x] - roff;
+  if (nrows_item <= 0) return;                   // the whole cluster leaves
+  const int nrows = nrows_item < MT * 16 ? nrows_item : MT * 16;
+  const int adapter = a.item_adapter[blockIdx.x];
+  const int32_t* rows = a.item_rows + a.item_start[blockIdx.x] + roff;
+  const int32_t* saves = a.item_save ? a.item_save + a.item_start[blockIdx.x] + roff : nullptr;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane >> 2, c = lane & 3;
+  const int CL = gridDim.y, ks = blockIdx.y;
+  const int nkb = a.D / 64;
+  const int kb_begin = (int)((long long)ks * nkb / CL), kb_end = (int)((long long)(ks + 1) * nkb / CL);
+
+  const __nv_bfloat16* xp[2 * MT];
+  __nv_bfloat16* sp[2 * MT];
+  int msave[2 * MT];             // DROP: save-order place of the row (the mask's row counter), -1: not a fine-tuning row
+#pragma unroll
+  for (int j = 0; j < 2 * MT; ++j) {
+    const int rl = g + 8 * j;
+    xp[j] = nullptr; sp[j] = nullptr; msave[j] = -1;
+    if (rl < nrows) {
+      const int row = rows[rl];
+      xp[j] = a.In + (size_t)row * a.ld_in + 16 * c;
+      const int sv = (saves && a.x_save && part == 0) ? saves[rl] : -1;
+      if (sv >= 0) sp[j] = a.x_save + (size_t)(a.save_base + sv) * a.D + 16 * c;
+      if (DROP && saves) msave[j] = saves[rl];
+    }
+  }
+  const __nv_bfloat16* Pa = a.P_all + ((size_t)adapter * R + q_base) * a.D;
+  for (int i = threadIdx.x; i < RP * (kb_end - kb_begin); i += FEW_WARPS * 32)
+    ptx::prefetch_l2(Pa + (size_t)(i % RP) * a.D + (size_t)(kb_begin + i / RP) * 64);
+  // table entries of the rows this warp finishes: rows ks + CL (warp + 4 i) of the CTA, lane i holds them
+  constexpr int FIN = MT * 16 / FEW_WARPS;       // most rows a warp finishes (cluster of one)
+  int f_row = -1, f_save = -1, f_slot = 0, f_cols = 0, f_c0 = 0, f_w = 0;   // operand: chunk slot, columns of the tile, the row's own [c0, c0 + w)
+  if (lane < FIN) {
+    const int r = ks + CL * (warp + FEW_WARPS * lane);
+    if (r < nrows) {
+      f_row = rows[r];
+      f_save = saves ? saves[r] : -1;
+      if (a.pbd.pbd) {
+        const int tile = f_row >> 8, goff = a.pbd.tile2_grp_off[tile], g = a.pbd.row_grp2[f_row];
+        f_slot = 2 * goff;
+        f_cols = a.pbd.tile2_cols ? a.pbd.tile2_cols[tile] : (a.pbd.tile2_grp_off[tile + 1] - goff) * R;
+        f_c0 = a.pbd.grp2_col ? a.pbd.grp2_col[goff + g] : g * R;
+        f_w = a.pbd.grp2_width ? a.pbd.grp2_width[goff + g] : R;
+      }
+    }
+  }
+  const __nv_bfloat16* p0 = Pa + (size_t)g * a.D + 16 * c;
+  // everything above read only the plan's tables; from here on the predecessor's data is touched
+  ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();
+  const float sc = a.scale ? a.scale[adapter] : 1.0f;
+  const float psc = a.pbd.pbd && a.pbd.scale ? a.pbd.scale[adapter] : 1.0f;
+  if (a.pbd.pbd && blockIdx.y == 0 && blockIdx.z == 0)         // rows nobody else owns: all-zero chunks
+    for (int i = blockIdx.x * FEW_WARPS + warp; i < a.pbd.n_zero_rows; i += gridDim.x * FEW_WARPS)
+      pbd_write_row<R>(a.pbd, a.pbd.zero_rows[i], nullptr, 0.f, lane);
+
+  float acc[MT][RB][4];
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int i = 0; i < RB; ++i) acc[m][i][0] = acc[m][i][1] = acc[m][i][2] = acc[m][i][3] = 0.f;
+  const uint4 zero4 = make_uint4(0, 0, 0, 0);
+#pragma unroll(RB * MT <= 4 ? 2 : 1)
+  for (int kb = kb_begin + warp; kb < kb_end; kb += FEW_WARPS) {
+    const int ko = kb * 64;
+    uint4 x[2 * MT][2];
+#pragma unroll
+    for (int j = 0; j < 2 * MT; ++j) {
+      x[j][0] = zero4; x[j][1] = zero4;
+      if (xp[j]) { x[j][0] = ptx::ldg_nc_v4(xp[j] + ko); x[j][1] = ptx::ldg_nc_v4(xp[j] + ko + 8); }
+    }
+    uint4 pa[RB], pb[RB];
+#pragma unroll
+    for (int i = 0; i < RB; ++i) {
+      const __nv_bfloat16* pp = p0 + (size_t)i * 8 * a.D + ko;
+      pa[i] = __ldg(reinterpret_cast<const uint4*>(pp));
+      pb[i] = __ldg(reinterpret_cast<const uint4*>(pp + 8));
+    }
+    // activation save: the rows pass through registers exactly once; the saved copy keeps them as they are
+#pragma unroll
+    for (int j = 0; j < 2 * MT; ++j) {
+      if (sp[j]) {
+        *reinterpret_cast<uint4*>(sp[j] + ko) = x[j][0];
+        *reinterpret_cast<uint4*>(sp[j] + ko + 8) = x[j][1];
+      }
+      if (DROP && msave[j] >= 0) {
+        drop_mask8(a.drop, (uint32_t)msave[j], (uint32_t)(ko + 16 * c), x[j][0]);
+        drop_mask8(a.drop, (uint32_t)msave[j], (uint32_t)(ko + 16 * c + 8), x[j][1]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < RB; ++i) {
+      const uint32_t rp[8] = {pa[i].x, pa[i].y, pa[i].z, pa[i].w, pb[i].x, pb[i].y, pb[i].z, pb[i].w};
+#pragma unroll
+      for (int m = 0; m < MT; ++m) {
+        const uint4 &l0 = x[2 * m][0], &l1 = x[2 * m][1], &h0 = x[2 * m + 1][0], &h1 = x[2 * m + 1][1];
+        const uint32_t ra[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
+        const uint32_t rb[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+          ptx::mma_bf16_16816(acc[m][i], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1], rp[2 * s], rp[2 * s + 1]);
+      }
+    }
+  }
+
+  // sum over the warps, in warp order
+#pragma unroll
+  for (int w = 0; w < FEW_WARPS; ++w) {
+    if (warp == w) {
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int i = 0; i < RB; ++i) {
+          float2* r0 = reinterpret_cast<float2*>(&sum[m * 16 + g][i * 8 + 2 * c]);
+          float2* r1 = reinterpret_cast<float2*>(&sum[m * 16 + g + 8][i * 8 + 2 * c]);
+          if (w == 0) {
+            *r0 = make_float2(acc[m][i][0], acc[m][i][1]);
+            *r1 = make_float2(acc[m][i][2], acc[m][i][3]);
+          } else {
+            const float2 u = *r0, v = *r1;
+            *r0 = make_float2(u.x + acc[m][i][0], u.y + acc[m][i][1]);
+            *r1 = make_float2(v.x + acc[m][i][2], v.y + acc[m][i][3]);
+          }
+        }
+    }
+    __syncthreads();
+  }
+  if (CL > 1) ptx::cluster_sync_all();
+  // sum over the cluster, in K order: one row per warp and turn
+  const uint32_t base = ptx::smem_u32(&sum[0][0]);
+  for (int i = 0; ks + CL * (warp + FEW_WARPS * i) < nrows; ++i) {
+    const int r = ks + CL * (warp + FEW_WARPS * i);
+    const int row = __shfl_sync(0xffffffffu, f_row, i), sv = __shfl_sync(0xffffffffu, f_save, i);
+    if (lane < RP) {
+      const uint32_t at = base + (uint32_t)(r * PITCH + lane) * 4u;
+      float parts[8];
+#pragma unroll
+      for (int s = 0; s < 8; ++s) parts[s] = s < CL ? (CL > 1 ? ld_cluster_f32(ptx::map_to_cta(at, (uint32_t)s)) : sum[r][lane]) : 0.f;
+      float u = 0.f;
+#pragma unroll
+      for (int s = 0; s < 8; ++s) u += parts[s];
+      if (DROP && sv >= 0) u *= a.drop.keep_scale;
+      a.Out[(size_t)row * R + q_base + lane] = u * sc;
+      if (a.u_save && sv >= 0) a.u_save[(size_t)(a.save_base + sv) * R + q_base + lane] = u;
+      fin[warp][lane] = u * sc;
+    }
+    __syncwarp();
+    if (a.pbd.pbd) {
+      // the row's operand chunks: this part's own columns; the zeros around the row's group come from part 0
+      const int slot = __shfl_sync(0xffffffffu, f_slot, i), cols = __shfl_sync(0xffffffffu, f_cols, i);
+      const int c0 = __shfl_sync(0xffffffffu, f_c0, i), w = __shfl_sync(0xffffffffu, f_w, i);
+      __nv_bfloat16* chunk0 = a.pbd.pbd + ((size_t)slot * 256 + (row & 255)) * 64;
+      for (int piece = lane; piece < (cols + 63) / 64 * 8; piece += 32) {
+        const int q = piece * 8 - c0;                       // rank of the piece's first column
+        const bool own = q >= 0 && q < w;
+        if (own ? q / RP != part : part != 0) continue;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (own) {
+          const float* f = &fin[warp][q - q_base];
+          v = make_uint4(ptx::pack_bf16(f[0] * psc, f[1] * psc), ptx::pack_bf16(f[2] * psc, f[3] * psc),
+                         ptx::pack_bf16(f[4] * psc, f[5] * psc), ptx::pack_bf16(f[6] * psc, f[7] * psc));
+        }
+        *reinterpret_cast<uint4*>(chunk0 + (size_t)(piece >> 3) * (256 * 64) + (piece & 7) * 8) = v;
+      }
+    }
+    __syncwarp();
+  }
+  if (CL > 1) ptx::cluster_sync_all();           // the peers have read this CTA's sums
+}
+
+// ---------------------------------------------------------------------------------------------
 // Streaming shrink for ranks up to 32: a persistent grid (one CTA per SM) walks the flattened list
 // of work units (item, chunk of 8 K-blocks = 512 elements) in equal contiguous ranges, so every SM
 // streams the same number of bytes in one wave.  A producer warp moves each unit into a

@@ -1,0 +1,104 @@
+"""Batches small enough for the few-row kernels (weight-streaming GEMM with its K slices summed inside a cluster, cluster
+shrink) at the sizes where their tiles and slices can go wrong: one row up to and beyond a row tile of 128, widths that leave
+a half-filled column tile, contractions with an odd number of K-blocks, every rank, plans with per-adapter ranks, strides."""
+import numpy as np
+import pytest
+
+from oracle import mlora_oracle as orc
+from paper_2607_28848_b200 import binding as mb
+from paper_2607_28848_b200 import synth
+from paper_2607_28848_b200.runner import LayerRun, Session
+from test_gpu_parity import TOL, assert_close, run_and_check
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sess():
+    s = Session(0)
+    yield s
+    s.close()
+
+
+# (rows, d_in, d_out): K slices 1 to 8; 320 = 2.5 column tiles; 576 and 1088 = an odd number of K-blocks; 300 and 700 rows =
+# row tiles of 128 with a remainder; 16384 -> 64: one half-filled column tile in eight slices
+SIZES = [(1, 576, 320), (16, 1024, 128), (17, 4096, 192), (64, 1088, 448), (65, 2048, 320), (128, 576, 1024), (129, 1088, 192),
+         (255, 512, 320), (256, 4096, 256), (300, 576, 448), (700, 1024, 320), (40, 16384, 64)]
+
+
+@pytest.mark.parametrize("rank", [8, 16, 32, 64, 128])
+@pytest.mark.parametrize("rows,d_in,d_out", SIZES)
+def test_few_rows(sess, rows, d_in, d_out, rank):
+    w = synth.random_workload(1000 + rows + rank, d_in, d_out, rank, 7, rows, max_seg=max(2, rows // 3), p_finetune=0.5)
+    run_and_check(sess, w, synth.make_tensors(w), blocked=True)
+
+
+@pytest.mark.parametrize("rank", [8, 64])
+def test_every_row_its_own_adapter(sess, rank):
+    """200 decode rows over 200 adapters: the low-rank operand is many times as deep as the contraction, an odd number of
+    groups falls into each row tile and each slice."""
+    segs = synth.segments_array([(i, 1, (7 * i) % 211, 0) for i in range(200)] + [(200, 30, 5, 1)])
+    w = synth.Workload("own_adapters", 512, 320, rank, 211, "bf16", 230, segs, seed=rank)
+    run_and_check(sess, w, synth.make_tensors(w), blocked=True)
+
+
+def test_rows_of_the_base_model_only(sess):
+    """No rank-r launch in front of the GEMM: it has to wait for whatever wrote its input."""
+    segs = synth.segments_array([(0, 50, -1, 0)])
+    w = synth.Workload("base_only", 1024, 320, 16, 3, "bf16", 50, segs, seed=3)
+    t = synth.make_tensors(w, with_grad=False)
+    ref = orc.forward(t["X"], t["W"], t["A_all"], t["B_all"], t["scale"], w.segments)["Y"]
+    run = LayerRun(sess, w.dtype, t, w.segments, w.n_rows)
+    try:
+        X = run.X.clone()
+        for _ in range(20):                         # the input is written by the launch right in front of the call
+            run.X.zero_()
+            run.X.add_(X)
+            run.forward()
+        assert run.status() == mb.MLORA_OK
+        assert_close("Y", run.host(run.Y), ref, TOL["bf16"])
+    finally:
+        run.close()
+
+
+@pytest.mark.parametrize("rows", [60, 230])
+def test_ranked_plans(sess, rows):
+    ranks = [16, 64, 32, 16, 48, 8, 16, 64, 24]
+    w = synth.random_workload(1300 + rows, 1024, 320, 64, len(ranks), rows, max_seg=12, p_decode=0.5, p_finetune=0.4)
+    t = synth.make_tensors(w)
+    for a, r in enumerate(ranks):
+        t["A_all"][a, r:] = 0
+        t["B_all"][a, r:] = 0
+    outs = []
+    for ar in (None, ranks):
+        run = LayerRun(sess, w.dtype, t, w.segments, w.n_rows, adapter_rank=ar)
+        try:
+            run.forward()
+            run.backward()
+            assert run.status() == mb.MLORA_OK
+            outs.append([run.host(b) for b in (run.Y, run.u_save, run.dX, run.dA, run.dB)])
+        finally:
+            run.close()
+    fwd = orc.forward(t["X"], t["W"], t["A_all"], t["B_all"], t["scale"], w.segments)
+    assert_close("Y", outs[1][0], fwd["Y"], TOL["bf16"])
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b)
+
+
+def test_slices_give_the_same_bits_every_time(sess):
+    """The cluster's sums are added in slice order, whoever is done first."""
+    w = synth.random_workload(1400, 8192, 512, 16, 5, 90, max_seg=20, p_finetune=0.5)
+    t = synth.make_tensors(w)
+    run = LayerRun(sess, w.dtype, t, w.segments, w.n_rows)
+    try:
+        first = None
+        for _ in range(5):
+            run.forward()
+            run.backward()
+            got = [run.host(b) for b in (run.Y, run.u_save, run.dX, run.dA, run.dB)]
+            if first is None:
+                first = got
+            assert all(np.array_equal(a, b) for a, b in zip(first, got))
+        assert run.status() == mb.MLORA_OK
+    finally:
+        run.close()
