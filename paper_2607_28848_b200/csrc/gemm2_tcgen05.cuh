@@ -19,6 +19,10 @@
 //   empty[s]      in each CTA: tcgen05.commit multicast to both (releases both producers).
 //   tmem_full[b]  in each CTA: tcgen05.commit multicast (wakes both epilogues).
 //   tmem_empty[b] in the leader: 8 arrivals = 4 epilogue warps x 2 CTAs.
+// With `early` set the main loop starts while the launch in front (the call's own shrink or gradient kernel) still drains:
+// neither operand comes from it, only the low-rank blocks do, and those are the last of a tile (see gemm_rows_tcgen05.cuh
+// for when the host may set it).  1600 rows 4096 -> 4096 forward + backward: 108.3 -> 106.0 us; 475 rows 2816 -> 10880 with
+// 227 fine-tuning rows: 90 -> 81 us; nothing at sizes where the power cap sets the clock.
 // Every wait is bounded; the pair leaves through a cluster barrier before tensor memory is freed,
 // so neither CTA exits while the other may still touch its shared memory.
 #pragma once
@@ -188,7 +192,7 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
   ptx::cluster_sync_all();                           // the peer's barriers exist from here on
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_ptr_smem;
-  ptx::grid_dependency_wait();
+  if (!args.early) ptx::grid_dependency_wait();
   ptx::grid_launch_dependents();
 
   const int KB = (args.K + GEMM_BK - 1) / GEMM_BK;
@@ -213,7 +217,7 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
     // the list costs one memory latency per tile rather than one per group.
     int32_t* ga_smem = reinterpret_cast<int32_t*>(smem_gen + (sMisc - smem_base) + 64);   // 256 entries
     uint32_t it = 0;
-    bool ok = true;
+    bool ok = true, waited = false;
     for (int ui = u_begin; ui < u_end && ok; ui += u_step) {
       const int unit = ulist ? ulist[ui] : ui;
       int tile, ks, SK;
@@ -253,6 +257,10 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
         if (!ok) break;
       }
       if (!ok) break;
+      if (lc_end > lc_begin && args.early && !waited) {      // the low-rank operand comes from the launch before
+        ptx::grid_dependency_wait();
+        waited = true;
+      }
       if (lc_end > lc_begin && !ranked) {
 #pragma unroll
         for (int j = 0; j < 8; ++j)
@@ -451,6 +459,8 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
     }
     if (lane == 0) ptx::tma_store_wait<0>();
     __syncwarp();
+    // no CTA ends before the launch ahead of it has: what follows in the stream may rely on that
+    ptx::grid_dependency_wait();
   }
 
   // ============================ common exit ============================

@@ -50,6 +50,7 @@ struct GemmArgs {
   int32_t n_full;                // work units [0, n_full) are whole 128 x 256 tiles; the tiles after
   int32_t n_units;               // them (the last, partly filled wave) are cut into two 128 x 128 halves
   int32_t lora_enabled;
+  int32_t early;                 // two-SM kernel only: In and the weight may be read before the dependency wait
   int32_t group_m;               // two-SM kernel only: row tiles per band of the tile order (0: one band)
   // Two-SM kernel only: tiles [0, n_whole) are whole work units; each of the n_tail tiles after them is
   // cut into split_k K slices (units after the whole ones, slice-major), whose fp32 partial tiles go
