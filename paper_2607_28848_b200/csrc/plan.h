@@ -79,17 +79,18 @@ inline void build_tile_groups(const std::vector<int32_t>& row_adapter, int32_t t
   row_grp.assign(n, -1);
   tile_grp_off.assign(1, 0);
   grp_adapter.clear();
+  // group of an adapter in the current tile: valid where the entry is not older than the tile's first group
+  int32_t max_adapter = -1;
+  for (int32_t a : row_adapter) max_adapter = a > max_adapter ? a : max_adapter;
+  std::vector<int32_t> last(max_adapter + 1, -1);
   for (int32_t t0 = 0; t0 < n; t0 += tile_rows) {
     const int32_t t1 = t0 + tile_rows < n ? t0 + tile_rows : n;
     const int32_t base = (int32_t)grp_adapter.size();
     for (int32_t t = t0; t < t1; ++t) {
       const int32_t a = row_adapter[t];
       if (a < 0) continue;
-      int32_t g = -1;
-      for (int32_t i = base; i < (int32_t)grp_adapter.size(); ++i)
-        if (grp_adapter[i] == a) { g = i - base; break; }
-      if (g < 0) { g = (int32_t)grp_adapter.size() - base; grp_adapter.push_back(a); }
-      row_grp[t] = g;
+      if (last[a] < base) { last[a] = (int32_t)grp_adapter.size(); grp_adapter.push_back(a); }
+      row_grp[t] = last[a] - base;
     }
     tile_grp_off.push_back((int32_t)grp_adapter.size());
   }
