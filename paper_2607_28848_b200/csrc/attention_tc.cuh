@@ -11,10 +11,10 @@
 //                                    into columns 256..383
 //   warps 2..9         softmax:      two threads per query row (warps w and w + 4 own the same 32 lanes of
 //                                    tensor memory), each with 64 of the block's 128 keys and 64 of the 128
-//                                    output columns.  A thread reads its half of S_j twice from tensor memory
-//                                    (row maximum - exchanged with its partner through shared memory behind an
-//                                    mbarrier of the warp pair - then exponentials), masks (same sequence,
-//                                    key <= query) and keeps P_j as packed bf16 in 32 registers; only then it
+//                                    output columns.  A thread reads its half of S_j from tensor memory,
+//                                    masks it where its warp has to (same sequence, key <= query), exchanges the
+//                                    row maximum with its partner through shared memory behind an mbarrier of
+//                                    the warp pair, takes the exponentials and keeps P_j as packed bf16 in 32 registers; only then it
 //                                    takes the previous block's O_blk into its 64 fp32 output registers,
 //                                    rescaled by exp2(m_old - m_new) (online softmax; nothing is rescaled in
 //                                    tensor memory), and writes P_j in the K-major swizzled operand layout -
@@ -26,6 +26,8 @@
 // out sets the CTA's abort flag and a device status word, and the CTA leaves through the common
 // exit that frees its tensor memory.
 #pragma once
+
+#include <type_traits>
 
 #include "gemm_tcgen05.cuh"
 #include "ptx.cuh"
@@ -226,38 +228,33 @@ forward_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       ok = __all_sync(0xffffffffu, gemm_wait(bar_s(j), (j >> 1) & 1, abort_flag, &g_status));   // one decision per warp:
       if (!ok) break;                                                                            // the loads below are warp-wide
       ptx::tc_fence_after();
-      float mx = m;
+      // the thread's 64 scores, read once (twice before, each behind its own wait); the masks cost as much as the
+      // exponentials, so a block that no row of the warp has to mask (most blocks of a long sequence) goes without them.
+      // 4 x 512 tokens, 32 heads: 50 -> 40 us, 1 x 2048 120 -> 80 us; the chain of latencies from S to P still bounds it
+      uint32_t v[64];
+      ptx::tmem_ld_32x32b_x32(tS, *reinterpret_cast<uint32_t(*)[32]>(v));
+      ptx::tmem_ld_32x32b_x32(tS + 32, *reinterpret_cast<uint32_t(*)[32]>(v + 32));
+      ptx::tmem_ld_wait();
+      if (!__all_sync(0xffffffffu, key0 >= my_start && key0 + 63 <= i_abs)) {
 #pragma unroll
-      for (int cc = 0; cc < 2; ++cc) {
-        uint32_t v[32];
-        ptx::tmem_ld_32x32b_x32(tS + cc * 32, v);
-        ptx::tmem_ld_wait();
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          const int col = key0 + cc * 32 + k;
-          const float sc = (col >= my_start && col <= i_abs) ? __uint_as_float(v[k]) * a.scale_log2 : -1e30f;
-          mx = fmaxf(mx, sc);
-        }
+        for (int k = 0; k < 64; ++k)
+          if (key0 + k < my_start || key0 + k > i_abs) v[k] = 0xff7fffffu;       // most negative float: weight 0 for every maximum
       }
-      float peer_mx;
+      float top = -3.0e38f;
+#pragma unroll
+      for (int k = 0; k < 64; ++k) top = fmaxf(top, __uint_as_float(v[k]));
+      float mx = fmaxf(m, top * a.scale_log2), peer_mx;
       if (!(ok = exchange(mx, j & 1, j, peer_mx))) break;
       mx = fmaxf(mx, peer_mx);
       const float alpha = fast_ex2(m - mx);
       float rowsum = 0.f;
       uint32_t pk[32];
 #pragma unroll
-      for (int cc = 0; cc < 2; ++cc) {
-        uint32_t v[32];
-        ptx::tmem_ld_32x32b_x32(tS + cc * 32, v);
-        ptx::tmem_ld_wait();
-#pragma unroll
-        for (int k = 0; k < 32; k += 2) {
-          const int col = key0 + cc * 32 + k;
-          const float p0 = (col >= my_start && col <= i_abs) ? fast_ex2(__uint_as_float(v[k]) * a.scale_log2 - mx) : 0.f;
-          const float p1 = (col + 1 >= my_start && col + 1 <= i_abs) ? fast_ex2(__uint_as_float(v[k + 1]) * a.scale_log2 - mx) : 0.f;
-          rowsum += p0 + p1;
-          pk[cc * 16 + (k >> 1)] = ptx::pack_bf16(p0, p1);
-        }
+      for (int k = 0; k < 64; k += 2) {
+        const float p0 = fast_ex2(__uint_as_float(v[k]) * a.scale_log2 - mx);
+        const float p1 = fast_ex2(__uint_as_float(v[k + 1]) * a.scale_log2 - mx);
+        rowsum += p0 + p1;
+        pk[k >> 1] = ptx::pack_bf16(p0, p1);
       }
       if (j > 0) {      // the previous block's P V ran while this block's scores were worked on
         ok = __all_sync(0xffffffffu, gemm_wait(bar_o, (j - 1) & 1, abort_flag, &g_status));
@@ -497,22 +494,27 @@ backward_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       ok = __all_sync(0xffffffffu, gemm_wait(bar_s, j & 1, abort_flag, &g_status));
       if (!ok) break;
       ptx::tc_fence_after();
+      auto write_ds = [&](auto masked) {
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        uint32_t vs[32], vp[32];
-        ptx::tmem_ld_32x32b_x32(tS + cc * 32, vs);
-        ptx::tmem_ld_32x32b_x32(tP + cc * 32, vp);
-        ptx::tmem_ld_wait();
-        uint32_t pk[16];
+        for (int cc = 0; cc < 4; ++cc) {
+          uint32_t vs[32], vp[32];
+          ptx::tmem_ld_32x32b_x32(tS + cc * 32, vs);
+          ptx::tmem_ld_32x32b_x32(tP + cc * 32, vp);
+          ptx::tmem_ld_wait();
+          auto weight = [&](int k) -> float {        // a masked pair counts nothing whatever its score and the row's lse are
+            const int col = key0 + cc * 32 + k;
+            if (decltype(masked)::value && (col < my_start || col > i_abs)) return 0.f;
+            return fast_ex2(__uint_as_float(vs[k]) * a.scale_log2 - lse2);
+          };
+          uint32_t pk[16];
 #pragma unroll
-        for (int k = 0; k < 32; k += 2) {
-          const int col = key0 + cc * 32 + k;
-          const float p0 = (col >= my_start && col <= i_abs) ? fast_ex2(__uint_as_float(vs[k]) * a.scale_log2 - lse2) : 0.f;
-          const float p1 = (col + 1 >= my_start && col + 1 <= i_abs) ? fast_ex2(__uint_as_float(vs[k + 1]) * a.scale_log2 - lse2) : 0.f;
-          pk[k >> 1] = ptx::pack_bf16(p0 * (__uint_as_float(vp[k]) - D), p1 * (__uint_as_float(vp[k + 1]) - D));
+          for (int k = 0; k < 32; k += 2)
+            pk[k >> 1] = ptx::pack_bf16(weight(k) * (__uint_as_float(vp[k]) - D), weight(k + 1) * (__uint_as_float(vp[k + 1]) - D));
+          store_row_chunk(sDS, row, cc, pk);
         }
-        store_row_chunk(sDS, row, cc, pk);
-      }
+      };
+      if (__all_sync(0xffffffffu, key0 >= my_start && key0 + BN - 1 <= i_abs)) write_ds(std::false_type());   // as in the forward
+      else write_ds(std::true_type());
       ptx::fence_proxy_async_smem();
       ptx::tc_fence_before();
       ptx::mbar_arrive(bar_ds);
@@ -646,14 +648,15 @@ backward_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       const int h = hk * rep + it / nqb, q0 = k0 + (it % nqb) * BM;
       ok = __all_sync(0xffffffffu, gemm_wait(bar_ld_full, it & 1, abort_flag, &g_status));
       if (!ok) break;
-      {   // query q0 + row: D from the staged dO and O rows (same swizzle, so piece by piece), lse, sequence start
+      {   // query q0 + row: D from the staged dO and O rows, lse, sequence start.  Lane by lane another piece of the 128 bytes
+          // (the operand's swizzle): read at one offset by every lane the rows fall into one bank group, 2 us per block.
         const int i = q0 + row;
         float D = 0.f;
 #pragma unroll
         for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
           for (int pz = 0; pz < 8; ++pz) {
-            const uint32_t off = (uint32_t)kb * 16384u + (uint32_t)row * 128u + (uint32_t)pz * 16u;
+            const uint32_t off = (uint32_t)kb * 16384u + (uint32_t)row * 128u + (uint32_t)(pz ^ (row & 7)) * 16u;
             uint4 x, y;
             asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "r"(sOP + off));
             asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(y.x), "=r"(y.y), "=r"(y.z), "=r"(y.w) : "r"(sdO + off));
@@ -677,35 +680,42 @@ backward_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       ok = __all_sync(0xffffffffu, gemm_wait(bar_s, it & 1, abort_flag, &g_status));
       if (!ok) break;
       ptx::tc_fence_after();
+      auto write_p_ds = [&](auto masked) {
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        uint32_t vs[32], vp[32];
-        ptx::tmem_ld_32x32b_x32(tS + cc * 32, vs);
-        ptx::tmem_ld_32x32b_x32(tP + cc * 32, vp);
-        ptx::tmem_ld_wait();
-        uint32_t pp[16], pd[16];
+        for (int cc = 0; cc < 4; ++cc) {
+          uint32_t vs[32], vp[32];
+          ptx::tmem_ld_32x32b_x32(tS + cc * 32, vs);
+          ptx::tmem_ld_32x32b_x32(tP + cc * 32, vp);
+          ptx::tmem_ld_wait();
+          uint32_t pp[16], pd[16];
 #pragma unroll
-        for (int k4 = 0; k4 < 32; k4 += 4) {       // the per-query tables come in as vectors, four columns at a time
-          const int c0 = cc * 32 + k4;
-          const float4 l4 = *reinterpret_cast<const float4*>(sL + c0);
-          const float4 d4 = *reinterpret_cast<const float4*>(sD + c0);
-          const int4 s4 = *reinterpret_cast<const int4*>(sQS + c0);
-          const float lv[4] = {l4.x, l4.y, l4.z, l4.w}, dv4[4] = {d4.x, d4.y, d4.z, d4.w};
-          const int sv[4] = {s4.x, s4.y, s4.z, s4.w};
-          float p[4];
+          for (int k4 = 0; k4 < 32; k4 += 4) {       // the per-query tables come in as vectors, four columns at a time
+            const int c0 = cc * 32 + k4;
+            const float4 l4 = *reinterpret_cast<const float4*>(sL + c0);
+            const float4 d4 = *reinterpret_cast<const float4*>(sD + c0);
+            const float lv[4] = {l4.x, l4.y, l4.z, l4.w}, dv4[4] = {d4.x, d4.y, d4.z, d4.w};
+            float p[4];
+            if (decltype(masked)::value) {
+              const int4 s4 = *reinterpret_cast<const int4*>(sQS + c0);
+              const int sv[4] = {s4.x, s4.y, s4.z, s4.w};
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const int i = q0 + c0 + t;
-            p[t] = (j_abs <= i && j_abs >= sv[t]) ? fast_ex2(__uint_as_float(vs[k4 + t]) * a.scale_log2 - lv[t]) : 0.f;
+              for (int t = 0; t < 4; ++t)
+                p[t] = (j_abs <= q0 + c0 + t && j_abs >= sv[t]) ? fast_ex2(__uint_as_float(vs[k4 + t]) * a.scale_log2 - lv[t]) : 0.f;
+            } else {
+#pragma unroll
+              for (int t = 0; t < 4; ++t) p[t] = fast_ex2(__uint_as_float(vs[k4 + t]) * a.scale_log2 - lv[t]);
+            }
+            pp[k4 >> 1] = ptx::pack_bf16(p[0], p[1]);
+            pp[(k4 >> 1) + 1] = ptx::pack_bf16(p[2], p[3]);
+            pd[k4 >> 1] = ptx::pack_bf16(p[0] * (__uint_as_float(vp[k4]) - dv4[0]), p[1] * (__uint_as_float(vp[k4 + 1]) - dv4[1]));
+            pd[(k4 >> 1) + 1] = ptx::pack_bf16(p[2] * (__uint_as_float(vp[k4 + 2]) - dv4[2]), p[3] * (__uint_as_float(vp[k4 + 3]) - dv4[3]));
           }
-          pp[k4 >> 1] = ptx::pack_bf16(p[0], p[1]);
-          pp[(k4 >> 1) + 1] = ptx::pack_bf16(p[2], p[3]);
-          pd[k4 >> 1] = ptx::pack_bf16(p[0] * (__uint_as_float(vp[k4]) - dv4[0]), p[1] * (__uint_as_float(vp[k4 + 1]) - dv4[1]));
-          pd[(k4 >> 1) + 1] = ptx::pack_bf16(p[2] * (__uint_as_float(vp[k4 + 2]) - dv4[2]), p[3] * (__uint_as_float(vp[k4 + 3]) - dv4[3]));
+          store_row_chunk(sOP, row, cc, pp);
+          store_row_chunk(sDS, row, cc, pd);
         }
-        store_row_chunk(sOP, row, cc, pp);
-        store_row_chunk(sDS, row, cc, pd);
-      }
+      };
+      if (__all_sync(0xffffffffu, j_abs <= q0 && j_abs >= sQS[BM - 1])) write_p_ds(std::false_type());     // starts ascend with the queries
+      else write_p_ds(std::true_type());
       ptx::fence_proxy_async_smem();
       ptx::tc_fence_before();
       ptx::mbar_arrive(bar_p);
