@@ -1151,7 +1151,7 @@ mlora_status_t simt_gemm(mlora_ctx* ctx, const T* In, int64_t ld_in, const T* W,
                          int N, int K, int R, int n_adapters, const DropArgs& drop, cudaStream_t st) {
   if (M <= 0) return MLORA_OK;
   if (cancelled(ctx)) return MLORA_CANCELLED;
-  dim3 grid((N + 31) / 32, (M + 31) / 32), block(32, 32);
+  const dim3 grid = simt::gemm_grid(M, N), block(32, simt::GEMM_ROWS);
   LaunchScope scope(ctx, st, KIND_SIMT);
   simt::gemm_lora_kernel<T, W_KMAJOR><<<grid, block, 0, st>>>(In, ld_in, W, ldw, L_all, P, scale, ds.row_adapter, Out,
                                                               ld_out, M, N, K, R, n_adapters, drop);
@@ -1242,7 +1242,7 @@ mlora_status_t forward_noalloc_t(const mlora_layer_t* L, const int32_t* row_adap
                                                  row_adapter, nullptr, scratch, (T*)nullptr, nullptr, 0, n_rows,
                                                  L->n_adapters, DropArgs{0, 0, 1.0f});
   if (cudaGetLastError() != cudaSuccess) return MLORA_ERR_CUDA;
-  dim3 grid((L->d_out + 31) / 32, (n_rows + 31) / 32), block(32, 32);
+  const dim3 grid = simt::gemm_grid(n_rows, L->d_out), block(32, simt::GEMM_ROWS);
   simt::gemm_lora_kernel<T, false><<<grid, block, 0, st>>>((const T*)X, ldx, (const T*)L->W, L->ldw,
                                                            (const T*)L->B_all, scratch, L->scale, row_adapter, (T*)Y,
                                                            ldy, n_rows, L->d_out, L->d_in, L->rank, L->n_adapters,

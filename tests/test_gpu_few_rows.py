@@ -102,3 +102,10 @@ def test_slices_give_the_same_bits_every_time(sess):
         assert run.status() == mb.MLORA_OK
     finally:
         run.close()
+
+
+@pytest.mark.parametrize("rows,d_in,d_out,rank", [(1, 33, 31, 4), (7, 97, 131, 5), (9, 256, 257, 8), (130, 511, 65, 16)])
+def test_fp32_tiles_of_eight_rows(sess, rows, d_in, d_out, rank):
+    """The fp32 product at row, column and contraction remainders of its 8 x 32 tiles and 32-deep blocks."""
+    w = synth.random_workload(1500 + rows, d_in, d_out, rank, 3, rows, dtype="f32", max_seg=max(2, rows // 2), p_finetune=0.5)
+    run_and_check(sess, w, synth.make_tensors(w))
