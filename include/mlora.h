@@ -210,6 +210,7 @@ mlora_status_t mlora_mixed_forward(mlora_ctx* ctx, const mlora_layer_t* layer, c
  *   dA      device [n_slots, rank, d_in]  fp32, dense (same orientation as A_all)
  *   dB      device [n_slots, rank, d_out] fp32, dense (same orientation as B_all)
  *   dX_ft   device [T_ft, d_in], row stride lddx, layer dtype; NULL skips dX
+ *           (may lie over x_save or u_save: both have been read before its first element is written)
  *   accumulate  0: dA, dB are overwritten;  nonzero: the new gradients are added to them
  * Slot g belongs to adapter mlora_plan_ft_adapters()[g]; several fine-tuning segments on one
  * adapter add into one slot.  A plan without fine-tuning rows makes this a no-op. */

@@ -382,6 +382,10 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
     const uint32_t stage0 = sEpi + (uint32_t)(warp - 2) * 8192u;
     uint32_t lt = 0;
     bool ok = true;
+    // Nothing is stored before the launch in front has ended: a tile without low-rank blocks waits for it nowhere else, and
+    // that launch may still read what lies under the output (dX over x_save).  No CTA ends before it either: what follows
+    // in the stream may rely on that.
+    if (args.early) ptx::grid_dependency_wait();
     for (int ui = u_begin; ui < u_end && ok; ui += u_step, ++lt) {
       const int unit = ulist ? ulist[ui] : ui;
       int tile, ks, SK;
@@ -459,8 +463,6 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
     }
     if (lane == 0) ptx::tma_store_wait<0>();
     __syncwarp();
-    // no CTA ends before the launch ahead of it has: what follows in the stream may rely on that
-    ptx::grid_dependency_wait();
   }
 
   // ============================ common exit ============================

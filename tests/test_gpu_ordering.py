@@ -1,0 +1,47 @@
+"""What the kernels that start beside the launch in front of them may touch before that launch has ended: their own operands,
+and nothing that it reads or writes.  Sizes of each GEMM path that starts early: the two-SM kernel with whole tiles and with
+every tile split along K, and the few-row kernel."""
+import pytest
+import torch
+
+from paper_2607_28848_b200 import binding as mb
+from paper_2607_28848_b200 import synth
+from paper_2607_28848_b200.runner import LayerRun, Session
+
+pytestmark = pytest.mark.gpu
+
+# (fine-tuning rows, d_in, d_out): input-gradient products of 3 x 16 whole tiles, 2 x 11 tiles in K slices, 8 few-row tiles
+DX_SIZES = [(700, 4096, 1024), (512, 2816, 10880), (120, 1024, 512)]
+
+
+@pytest.fixture(scope="module")
+def sess():
+    s = Session(0)
+    yield s
+    s.close()
+
+
+@pytest.mark.parametrize("rank", [16, 64])
+@pytest.mark.parametrize("dropout", [0.0, 0.3])
+@pytest.mark.parametrize("rows,d_in,d_out", DX_SIZES)
+def test_dx_over_the_saved_input(sess, rows, d_in, d_out, dropout, rank):
+    """dX in the memory of x_save: the gradient kernel in front has read x_save before the first element of dX is stored, also
+    where a tile has no low-rank blocks (under dropout none has).  Same bits as with buffers of their own."""
+    segs = synth.segments_array([(0, rows // 2, 0, 1), (rows // 2, rows - rows // 2, 2, 1)])
+    w = synth.Workload("dx_over_x_save", d_in, d_out, rank, 3, "bf16", rows, segs, seed=rows + rank)
+    run = LayerRun(sess, w.dtype, synth.make_tensors(w), w.segments, w.n_rows)
+    mb.mlora_set_dropout(sess.ctx, dropout, 77)
+    try:
+        run.forward()
+        run.backward()
+        want = [b.clone() for b in (run.dX, run.dA, run.dB)]
+        saved = run.x_save.clone()
+        run.dX = run.x_save
+        for _ in range(10):
+            run.x_save.copy_(saved)
+            run.backward()
+            assert all(torch.equal(a, b) for a, b in zip(want, (run.x_save, run.dA, run.dB)))
+        assert run.status() == mb.MLORA_OK
+    finally:
+        mb.mlora_set_dropout(sess.ctx, 0.0, 0)
+        run.close()
