@@ -217,7 +217,7 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
     // the list costs one memory latency per tile rather than one per group.
     int32_t* ga_smem = reinterpret_cast<int32_t*>(smem_gen + (sMisc - smem_base) + 64);   // 256 entries
     uint32_t it = 0;
-    bool ok = true, waited = false;
+    bool ok = true;
     for (int ui = u_begin; ui < u_end && ok; ui += u_step) {
       const int unit = ulist ? ulist[ui] : ui;
       int tile, ks, SK;
@@ -257,10 +257,10 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
         if (!ok) break;
       }
       if (!ok) break;
-      if (lc_end > lc_begin && args.early && !waited) {      // the low-rank operand comes from the launch before
-        ptx::grid_dependency_wait();
-        waited = true;
-      }
+      // The low-rank operand comes from the launch before.  Every role waits for that launch behind the first main loop, low-rank
+      // blocks or not: from here on a slot may come free, or an accumulator be read, only after it, and how long it takes
+      // must not count against the limit of a wait inside this kernel.
+      if (args.early && ui == u_begin) ptx::grid_dependency_wait();
       if (lc_end > lc_begin && !ranked) {
 #pragma unroll
         for (int j = 0; j < 8; ++j)
@@ -354,6 +354,7 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
           ptx::umma2_commit_both(bar_empty(s));
         }
         if (!ok) break;
+        if (args.early && ui == u_begin) ptx::grid_dependency_wait();      // as the producer
         const int LC = (lcols + 63) / 64;
         const int lc_begin = (int)((long long)ks * LC / SK), lc_end = (int)((long long)(ks + 1) * LC / SK);
         for (int lc = lc_begin; lc < lc_end; ++lc, ++it) {

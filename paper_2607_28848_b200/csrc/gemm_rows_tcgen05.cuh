@@ -169,7 +169,10 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
     asm volatile("bar.sync 1, 160;" ::: "memory");
     lora_range();
     const int box_begin = col_begin / box, box_end = (col_end + box - 1) / box;
+    int fills = 0;
     for (int lc = col_begin / 64; lc * 64 < col_end && ok; lc += KW, at.next()) {
+      // From the second lap on a slot comes free as the MMA warp goes through low-rank blocks, which wait for the launch before.
+      if (args.early && fills++ == S) ptx::grid_dependency_wait();
       if (lane == 0) ok = gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status);
       ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!ok) break;
@@ -244,6 +247,8 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
     asm volatile("bar.sync 4, 160;" ::: "memory");
     lora_range();
     if (lane == 0) {
+      // How long the launch before takes must not count against the limit of the waits below.
+      if (args.early && col_begin < col_end) ptx::grid_dependency_wait();
       // boxes of [2 halves][BOX rows][64 columns]: 16 operand columns are 16 rows of one box, or two boxes of 8
       auto lora_mma = [&](auto box_rows) {
         constexpr int BOX = decltype(box_rows)::value;
@@ -305,10 +310,11 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
       ptx::prefetch_l2(p);
       if (n0 + 64 < args.N) ptx::prefetch_l2(p + 64);
     }
+    // The MMAs of the low-rank blocks wait for the launch before, so its time must not count against the limit of the wait
+    // here.  And no CTA stores or ends before that launch has ended: what follows in the stream may rely on that.
+    ptx::grid_dependency_wait();
     gemm_wait(bar_done, 0, abort_flag, args.status);
     ptx::tc_fence_after();
-    // no CTA ends before the launch ahead of it has: what follows in the stream may rely on that
-    ptx::grid_dependency_wait();
   }
   __syncwarp();
 
