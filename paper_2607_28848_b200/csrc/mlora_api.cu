@@ -880,16 +880,18 @@ mlora_status_t launch_gemm(mlora_ctx* ctx, int R, const CUtensorMap& tIn, const 
 // (each pair's units then in tile order).  The list is made once per plan and shape on the host and
 // copied behind the plan's tables; g.unit_list stays null when round robin is within 3% of it, when the
 // plan reserved no room (even row spaces), or when the stream is being captured before the list exists.
-void balanced_units(mlora_ctx* ctx, const RowSpace& hs, const DevRowSpace& ds, int R, int kblocks, GemmArgs& g,
+// True: the list's copy, or the wait for it, was queued on `st`, so the launch in front of the GEMM is no longer a kernel.
+bool balanced_units(mlora_ctx* ctx, const RowSpace& hs, const DevRowSpace& ds, int R, int kblocks, GemmArgs& g,
                     cudaStream_t st) {
   g.unit_list = nullptr; g.sched_pairs = 0;
   SchedCache* sc = ds.sched;
-  if (!sc || !sc->dev || !sc->mirror || ctx->no_unit_lists || !g.lora_enabled) return;
-  if ((int64_t)sc->lc_spread * R < 2 * 64) return;          // tiles differ by less than two K-blocks
+  if (!sc || !sc->dev || !sc->mirror || ctx->no_unit_lists || !g.lora_enabled) return false;
+  if ((int64_t)sc->lc_spread * R < 2 * 64) return false;          // tiles differ by less than two K-blocks
   const int pairs = g.n_units < ctx->sm_count / 2 ? g.n_units : ctx->sm_count / 2;
-  if (pairs < 2 || g.n_units + pairs + 1 > kSchedCap) return;
+  if (pairs < 2 || g.n_units + pairs + 1 > kSchedCap) return false;
   std::lock_guard<std::mutex> lock(sc->mu);
   SchedEntry* e = nullptr;
+  bool queued = false;
   int slot = 0;
   for (; slot < sc->n; ++slot) {
     SchedEntry& x = sc->e[slot];
@@ -897,9 +899,9 @@ void balanced_units(mlora_ctx* ctx, const RowSpace& hs, const DevRowSpace& ds, i
         x.n_tail == g.n_tail && x.split_k == g.split_k && x.group_m == g.group_m) { e = &x; break; }
   }
   if (!e) {
-    if (sc->n >= kSchedSlots) return;
+    if (sc->n >= kSchedSlots) return false;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) { cudaGetLastError(); return; }
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) { cudaGetLastError(); return false; }
     // cost of every unit in K-blocks (+2: accumulator hand-over and the first loads of a tile)
     std::vector<int32_t> cost(g.n_units);
     for (int u = 0; u < g.n_units; ++u) {
@@ -954,18 +956,21 @@ void balanced_units(mlora_ctx* ctx, const RowSpace& hs, const DevRowSpace& ds, i
         e->use = false;
       }
       e->stream = st;
+      queued = true;
     }
     sc->n++;
   }
-  if (!e->use) return;
+  if (!e->use) return queued;
   if (e->stream != st && e->filled) {        // another stream than the one that filled the list: order behind the copy
     if (cudaEventQuery(e->filled) != cudaSuccess) {
       cudaGetLastError();
-      if (cudaStreamWaitEvent(st, e->filled, 0) != cudaSuccess) { cudaGetLastError(); return; }
+      queued = true;
+      if (cudaStreamWaitEvent(st, e->filled, 0) != cudaSuccess) { cudaGetLastError(); return queued; }
     }
   }
   g.unit_list = sc->dev + (size_t)slot * kSchedCap;
   g.sched_pairs = e->pairs;
+  return queued;
 }
 
 // A plan made with per-adapter ranks serves layers whose padded rank is a multiple of 16 and at least every adapter's own.
@@ -1099,7 +1104,7 @@ mlora_status_t gemm_bf16(mlora_ctx* ctx, const mlora_layer_t* L, const RowSpace&
     g.row_grp = ds.row_grp2; g.row_adapter = ds.row_adapter;
     g.tile_grp_off = ds.tile2_grp_off; g.grp_adapter = ds.grp2_adapter;
     g.P = P; g.scale = scale; g.status = ctx->status_dev;
-    balanced_units(ctx, hs, ds, R, kblocks, g, st);
+    if (balanced_units(ctx, hs, ds, R, kblocks, g, st)) g.early = 0;      // early: only right behind a kernel of this call
     CUtensorMap tPbd;
     const uint64_t slots = g.lora_enabled ? 2 * (uint64_t)hs.grp2_adapter.size() : 1;
     if ((s = make_tmap_bf16(ctx, &tPbd, ctx->ws_pbd ? (const void*)ctx->ws_pbd : In, 64, slots * 256, 64, 64, 128)) != MLORA_OK)

@@ -45,3 +45,36 @@ def test_dx_over_the_saved_input(sess, rows, d_in, d_out, dropout, rank):
     finally:
         mb.mlora_set_dropout(sess.ctx, 0.0, 0)
         run.close()
+
+
+@pytest.mark.parametrize("rank", [16, 64])
+@pytest.mark.parametrize("rows,d_in,d_out", [(700, 1024, 4096), (512, 10880, 2816), (120, 512, 1024), (200, 4096, 512)])
+def test_operands_written_by_the_launch_in_front_of_the_call(sess, rows, d_in, d_out, rank):
+    """Every operand of forward and backward is rewritten right in front of the call, two sets in turn: a kernel that starts
+    early must not see the set before.  The first pass over a new plan, which may make a unit list, is one of them."""
+    w = synth.random_workload(50 + rows + rank, d_in, d_out, rank, 5, rows, max_seg=rows // 3, p_finetune=0.6)
+    run = LayerRun(sess, w.dtype, synth.make_tensors(w), w.segments, w.n_rows)
+    operands = (run.X, run.W, run.A_all, run.B_all, run.dY)
+    sets = [[b.clone() for b in operands], [b.flip(0).clone() for b in operands]]
+    outs = (run.Y, run.x_save, run.u_save, run.dX, run.dA, run.dB)
+    want = []
+    try:
+        for s in sets:
+            for b, v in zip(operands, s):
+                b.copy_(v)
+            torch.cuda.synchronize()
+            run.forward()
+            torch.cuda.synchronize()
+            run.backward()
+            torch.cuda.synchronize()
+            want.append([b.clone() for b in outs])
+        for i in range(20):
+            for b, v in zip(operands, sets[i & 1]):
+                b.copy_(v)
+            run.forward()
+            run.dY.copy_(sets[i & 1][4])
+            run.backward()
+            assert all(torch.equal(a, b) for a, b in zip(want[i & 1], outs))
+        assert run.status() == mb.MLORA_OK
+    finally:
+        run.close()
