@@ -25,6 +25,7 @@
 
 #include "gemm_tcgen05.cuh"
 #include "ptx.cuh"
+#include "ring.h"
 
 namespace mlora {
 namespace rows {
@@ -65,14 +66,6 @@ __host__ __device__ __forceinline__ uint32_t smem_bytes(int nb, int kw, int stag
   const uint32_t ring = stage_bytes(nb, kw) * (uint32_t)stages, sums = (uint32_t)(slice_rows(nb, slices) * slices) * 1024u;
   return (ring > sums ? ring : sums) + 1024u;
 }
-
-// Place in the ring: slot and the parity of its current use.
-struct Ring {
-  int n, slot = 0;
-  uint32_t parity = 0;
-  __device__ explicit Ring(int stages) : n(stages) {}
-  __device__ __forceinline__ void next() { if (++slot == n) { slot = 0; parity ^= 1; } }
-};
 
 // Shared memory of this CTA -> shared memory of a CTA of the cluster, bytes counted on a barrier of that CTA.
 __device__ __forceinline__ void bulk_to_cta(uint32_t dst_cluster, uint32_t src, uint32_t bytes, uint32_t bar_cluster) {
@@ -143,9 +136,12 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
   // operand, both multiples of 16 but for the end of an odd number of groups of rank 8.
   int col_begin = 0, col_end = 0, grp0 = 0;
   auto lora_range = [&]() { col_begin = lora_info[0]; col_end = lora_info[1]; grp0 = lora_info[2]; };
-  // A producer that gives up lets its loads in flight land (bounded: the other producer may not have filled the slot).
+  // A producer that gives up lets its loads in flight land: the barrier of every slot it has filled, at the parity of that
+  // fill (bounded: the other producer may not have filled the slot).
   auto drain = [&](const Ring& at) {
-    for (uint32_t i = 0; i < (1u << 12) && !ptx::mbar_try_wait(bar_full(at.slot), at.parity); ++i) {}
+    at.last_uses([&](int slot, uint32_t parity) {
+      for (uint32_t i = 0; i < (1u << 12) && !ptx::mbar_try_wait(bar_full(slot), parity); ++i) {}
+    });
   };
   const int box = args.piece_src ? 16 : (args.R < 64 ? args.R : 64);      // rows of an adapter's matrix per low-rank load
   const int per = 64 / box;
@@ -166,6 +162,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
     ok = __shfl_sync(0xffffffffu, ok, 0);
     at.slot = __shfl_sync(0xffffffffu, at.slot, 0);
     at.parity = __shfl_sync(0xffffffffu, at.parity, 0);
+    at.used = __shfl_sync(0xffffffffu, at.used, 0);
     asm volatile("bar.sync 1, 160;" ::: "memory");
     lora_range();
     const int box_begin = col_begin / box, box_end = (col_end + box - 1) / box;
