@@ -355,6 +355,47 @@ const int* rows_clusters(const mlora_ctx* ctx) {
   return clusters;
 }
 
+// How the two-SM GEMM cuts an [M, K] x [K, N] product: its tiles, and the K slices of the last n_tail of them (1: none).
+// Few tiles for the CTA pairs there are (small batches, the backward of one 256-token fine-tuning batch): K is cut into slices
+// of at least 16 K-blocks that run on different pairs; the fp32 partials are summed by a small kernel afterwards (≈8 µs with
+// its launch, hence the bound on what the split has to save).
+struct PairSplit { int tiles, sk, n_tail; };
+PairSplit pair_split(const mlora_ctx* ctx, int M, int N, int K) {
+  const int tiles = ((M + GEMM2_BM - 1) / GEMM2_BM) * ((N + GEMM2_BN - 1) / GEMM2_BN);
+  const int pairs = ctx->sm_count / 2, kblocks = (K + GEMM_BK - 1) / GEMM_BK;
+  const size_t tile_ws = (size_t)GEMM2_BM * GEMM2_BN * sizeof(float);
+  int sk = 1, n_tail = 0;
+  if (2 * tiles <= pairs && kblocks >= 64 && !ctx->no_split_k) {          // every tile is split
+    sk = pairs / tiles;
+    sk = sk < kblocks / 16 ? sk : kblocks / 16;
+    sk = sk < 8 ? sk : 8;
+    n_tail = tiles;
+    // the same bound as for the last wave below (4096 -> 4096 backward of 256 rows, 16 tiles in
+    // four slices: 42.6 -> 36.3 µs for the whole call; two slices of such a product do not pay)
+    if (sk < 2 || (int64_t)kblocks * (sk - 1) < 40 * (int64_t)sk) { sk = 1; n_tail = 0; }
+  } else if (tiles > pairs && !ctx->no_split_k) {
+    // More tiles than CTA pairs, and the last wave fills at most half of them: only its tiles are
+    // cut along K (slices of at least 16 K-blocks), so that the wave takes 1 / slices of a tile's
+    // time.  E.g. 160 tiles on 74 pairs: 12 tail tiles in 6 slices, 2.17 instead of 3 tile times.
+    const int rem = tiles % pairs;
+    if (rem > 0 && 2 * rem <= pairs && kblocks >= 32) {
+      sk = pairs / rem;
+      sk = sk < kblocks / 16 ? sk : kblocks / 16;
+      sk = sk < 8 ? sk : 8;
+      n_tail = rem;
+      // Worth it only if the K-blocks the last wave no longer waits for (≈0.4 µs each) outweigh the
+      // reduction kernel and the fp32 partial traffic (≈8 µs): the bound below keeps out e.g. a
+      // 4096-deep product with a half-full last wave (two slices: 103 -> 101 + 8.6 µs) and lets in
+      // a 4096-deep one with 8 tail tiles in four slices (330 -> 314 + 7.7 µs) and the 14336-deep
+      // ones (343 -> 305 + 8.6 µs; 13824-deep with 12 tail tiles 255 -> 177 + 8.7 µs).
+      if (sk < 2 || (int64_t)kblocks * (sk - 1) < 40 * (int64_t)sk) { sk = 1; n_tail = 0; }
+    }
+  }
+  while (sk > 1 && (size_t)sk * n_tail * tile_ws > kSplitKBytes) --sk;
+  if (sk <= 1) { sk = 1; n_tail = 0; }
+  return {tiles, sk, n_tail};
+}
+
 // Rows of a tile, K-blocks per stage and K slices of the few-row GEMM for an [M, K] x [K, N] product, or false: the two-SM
 // kernel's product.  Measured on B200 (whole forward calls, 4 adapters of rank 16, two-SM path / this one, us):
 //   4096 -> 4096:   16 rows 21.3 / 12.8, 64 24.3 / 14.2, 128 27.2 / 16.2, 256 28.2 / 20.9, 512 35.7 / 29.1
@@ -366,23 +407,61 @@ const int* rows_clusters(const mlora_ctx* ctx) {
 // Slices: as many as clusters of that size are resident at once, with at least 8 K-blocks each.  Clusters of 3, 5 and 7
 // straddle SM pairs and do not all find room while the launch in front still holds SMs (44 of 45 clusters of 3: 28 us in a
 // row of launches of its own kind, 39 behind the streaming shrink), so those count for nine tenths.
+// Beside the two-SM kernel: every row tile runs all low-rank blocks of its 256-row tile, so a batch of many adapters, or one
+// whose K the two-SM kernel cuts finer, can be the worse here (4096 -> 4096, 256 rows of 256 adapters, two-SM / this, us: rank
+// 64 100 / 131, rank 128 153 / 210; 8192 -> 1024, 768 rows of rank 16 31.6 / 34).  The K-blocks behind one another decide, in
+// units of the two-SM kernel's 0.4 us, as fitted to 5600 forward and backward calls (8 to 3072 rows, ranks 8 to 128, 1 to 256
+// adapters, 11 shapes): 0.8 for a main block here, 1.1 for a low-rank one, 14 for the reduction launch behind a two-SM
+// product in K slices.  The choice is within 5% of the better one on 94% of them, and behind the two-SM kernel by more than
+// 3% on 3% (without it 9%, by up to 2.0x).
 struct RowsShape { int nb, kw, slices; };
-bool rows_shape(const mlora_ctx* ctx, int M, int N, int K, RowsShape& r) {
+bool rows_shape(const mlora_ctx* ctx, int M, int N, int K, int lr_cols, RowsShape& r) {
   if (ctx->gemm_path != 0 || ctx->shrink_path != 0 || !ctx->gemm_pairs || ctx->no_split_k || ctx->grad_mode != 0) return false;
   r.nb = M <= 128 ? (M + 15) / 16 * 16 : (M <= 256 ? ((M + 1) / 2 + 15) / 16 * 16 : 128);
   const int64_t tiles = (int64_t)((N + rows::BM - 1) / rows::BM) * ((M + r.nb - 1) / r.nb);
   if (tiles > ctx->sm_count) return false;
   const int* clusters = rows_clusters(ctx);
   if (!clusters) return false;
-  const int kblocks = K / GEMM_BK;
+  const int kblocks = K / GEMM_BK, lc = (lr_cols + 63) / 64;
   r.slices = 1;
   for (int c = 2; c <= 8; ++c)
     if (kblocks / c >= 8 && tiles <= ((c & 1) ? clusters[c] * 9 / 10 : clusters[c])) r.slices = c;
   r.kw = r.nb <= 64 ? 2 : 1;
-  return r.nb <= 64 || kblocks / r.slices <= 64;
+  if (r.nb > 64 && kblocks / r.slices > 64) return false;
+  const PairSplit two = pair_split(ctx, M, N, K);
+  const int pairs = ctx->sm_count / 2, whole = two.tiles - two.n_tail;
+  const float two_blocks = (float)(kblocks + lc) * ((float)((whole + pairs - 1) / pairs) + (two.n_tail > 0 ? 1.0f / two.sk : 0.f)) +
+                           (two.sk > 1 ? 14.f : 0.f);
+  return (0.8f * kblocks + 1.1f * lc) / r.slices <= two_blocks + 4.f;
+}
+// Columns of the low-rank operand of the fullest 256-row tile, by the layer's rank also for a plan with ranks of its own: both
+// kinds of plan take the same kernels and give the same bits.
+int lowrank_columns(const RowSpace& hs, int R) {
+  int32_t most = 0;
+  for (size_t t = 0; t + 1 < hs.tile2_grp_off.size(); ++t) {
+    const int32_t n = hs.tile2_grp_off[t + 1] - hs.tile2_grp_off[t];
+    most = n > most ? n : most;
+  }
+  return most * R;
 }
 
-// Shrink of a batch of few rows: items x a cluster along K, as many CTAs as two per SM.
+// CTAs along K per item of the few-row shrink: with the items, as many as two per SM.
+int few_cluster(const mlora_ctx* ctx, int R, int D, int n_items) {
+  const int parts = R > 32 ? R / 32 : 1, nkb = D / 64;
+  int cl = 1;
+  while (cl < 8 && cl * n_items * parts <= ctx->sm_count && nkb >= 2 * cl * FEW_WARPS) cl *= 2;
+  return cl;
+}
+// Whether that kernel is the faster one.  Many items leave it no CTAs along K, and its warps then wait for memory K-block after
+// K-block, which the kernels for larger batches do not: 32 (rank 8), 16, 8, 8 and 4 (rank 128) K-blocks per warp are where the
+// two meet in the forward.  At rank 128, 64 rows of 64 adapters, 8192 -> 2048 (32 K-blocks per warp) take 97 us with it and 58
+// without; 96 rows of one adapter, 14336 -> 4096 (eight CTAs along K, as many as there can be) 30 with it and 44 without.
+bool shrink_few_fits(const mlora_ctx* ctx, int R, int D, int n_items) {
+  const int cl = few_cluster(ctx, R, D, n_items), per_warp = (D / 64 + cl * FEW_WARPS - 1) / (cl * FEW_WARPS);
+  return cl == 8 || per_warp <= (R <= 32 ? 256 / R : (R <= 64 ? 8 : 4));
+}
+
+// Shrink of a batch of few rows: items x a cluster along K.
 template <int R, int MT, bool DROP>
 mlora_status_t launch_shrink_few_d(mlora_ctx* ctx, const ShrinkArgs& a, int n_items, cudaStream_t st) {
   static bool attr_set_dev[kMaxDevices] = {};   // per instantiation and device
@@ -395,9 +474,7 @@ mlora_status_t launch_shrink_few_d(mlora_ctx* ctx, const ShrinkArgs& a, int n_it
       attr_set_dev[ctx->device] = true;
     }
   }
-  const int parts = R > 32 ? R / 32 : 1, z = parts * (kItemRows / (16 * MT)), nkb = a.D / 64;
-  int cl = 1;
-  while (cl < 8 && cl * n_items * parts <= ctx->sm_count && nkb >= 2 * cl * FEW_WARPS) cl *= 2;
+  const int parts = R > 32 ? R / 32 : 1, z = parts * (kItemRows / (16 * MT)), cl = few_cluster(ctx, R, a.D, n_items);
   if (cancelled(ctx)) return MLORA_CANCELLED;
   LaunchScope scope(ctx, st, KIND_SHRINK);
   launch_pdl_cluster(scope.slot < 0, kern, dim3(n_items, cl, z), dim3(FEW_WARPS * 32), dim3(1, cl, 1), 0, st, a);
@@ -1030,7 +1107,7 @@ mlora_status_t gemm_bf16(mlora_ctx* ctx, const mlora_layer_t* L, const RowSpace&
                          const void* In, int64_t ld_in, void* Out, int64_t ld_out, const void* L_all,
                          const float* P, const float* scale, int M, int N, int K, cudaStream_t st, bool early, bool lora = true) {
   RowsShape shape;
-  if (rows_shape(ctx, M, N, K, shape)) {
+  if (rows_shape(ctx, M, N, K, lora ? lowrank_columns(hs, L->rank) : 0, shape)) {
     auto launch = shape.kw == 2 ? launch_gemm_rows<W_KMAJOR, 2> : launch_gemm_rows<W_KMAJOR, 1>;
     return launch(ctx, L, hs, ds, In, ld_in, Out, ld_out, L_all, M, N, K, shape, lora, early, st);
   }
@@ -1060,44 +1137,12 @@ mlora_status_t gemm_bf16(mlora_ctx* ctx, const mlora_layer_t* L, const RowSpace&
   if (ctx->gemm_pairs) {            // two-SM kernel: 256-row tiles and their group tables
     g.n_mtiles = (M + GEMM2_BM - 1) / GEMM2_BM;
     g.n_ntiles = (N + GEMM2_BN - 1) / GEMM2_BN;
-    // Few tiles for the CTA pairs there are (small batches, the backward of one 256-token fine-tuning
-    // batch): cut K into slices of at least 16 K-blocks that run on different pairs; the fp32 partials
-    // are summed by a small kernel afterwards (≈8 µs with its launch, hence the bound on what the split
-    // has to save).
     const int tiles = g.n_mtiles * g.n_ntiles, pairs = ctx->sm_count / 2, kblocks = (K + GEMM_BK - 1) / GEMM_BK;
     // The start beside the draining launch in front pays where that launch is a visible part of the time: up to two waves of
     // tiles (figures in gemm2_tcgen05.cuh); 896 tiles under the power cap measured 0.5% faster and 1.5% slower in two runs.
     g.early = early && tiles <= 2 * pairs ? 1 : 0;
-    const size_t tile_ws = (size_t)GEMM2_BM * GEMM2_BN * sizeof(float);
-    int sk = 1, n_tail = 0;
-    if (2 * tiles <= pairs && kblocks >= 64 && !ctx->no_split_k) {          // every tile is split
-      sk = pairs / tiles;
-      sk = sk < kblocks / 16 ? sk : kblocks / 16;
-      sk = sk < 8 ? sk : 8;
-      n_tail = tiles;
-      // the same bound as for the last wave below (4096 -> 4096 backward of 256 rows, 16 tiles in
-      // four slices: 42.6 -> 36.3 µs for the whole call; two slices of such a product do not pay)
-      if (sk < 2 || (int64_t)kblocks * (sk - 1) < 40 * (int64_t)sk) { sk = 1; n_tail = 0; }
-    } else if (tiles > pairs && !ctx->no_split_k) {
-      // More tiles than CTA pairs, and the last wave fills at most half of them: only its tiles are
-      // cut along K (slices of at least 16 K-blocks), so that the wave takes 1 / slices of a tile's
-      // time.  E.g. 160 tiles on 74 pairs: 12 tail tiles in 6 slices, 2.17 instead of 3 tile times.
-      const int rem = tiles % pairs;
-      if (rem > 0 && 2 * rem <= pairs && kblocks >= 32) {
-        sk = pairs / rem;
-        sk = sk < kblocks / 16 ? sk : kblocks / 16;
-        sk = sk < 8 ? sk : 8;
-        n_tail = rem;
-        // Worth it only if the K-blocks the last wave no longer waits for (≈0.4 µs each) outweigh the
-        // reduction kernel and the fp32 partial traffic (≈8 µs): the bound below keeps out e.g. a
-        // 4096-deep product with a half-full last wave (two slices: 103 -> 101 + 8.6 µs) and lets in
-        // a 4096-deep one with 8 tail tiles in four slices (330 -> 314 + 7.7 µs) and the 14336-deep
-        // ones (343 -> 305 + 8.6 µs; 13824-deep with 12 tail tiles 255 -> 177 + 8.7 µs).
-        if (sk < 2 || (int64_t)kblocks * (sk - 1) < 40 * (int64_t)sk) { sk = 1; n_tail = 0; }
-      }
-    }
-    while (sk > 1 && (size_t)sk * n_tail * tile_ws > kSplitKBytes) --sk;
-    if (sk <= 1) { sk = 1; n_tail = 0; }
+    const PairSplit split = pair_split(ctx, M, N, K);
+    const int sk = split.sk, n_tail = split.n_tail;
     g.split_k = sk; g.n_tail = n_tail; g.n_whole = tiles - n_tail; g.ws_splitk = ctx->ws_splitk;
     g.n_full = g.n_units = g.n_whole + n_tail * sk;
     g.lora_enabled = (lora && !hs.grp2_adapter.empty()) ? 1 : 0;
@@ -1698,7 +1743,8 @@ mlora_status_t mlora_mixed_forward(mlora_ctx* ctx, const mlora_layer_t* L, const
   // (a batch of few rows: the latency-bound shrink that its GEMM overlaps with; 10880 -> 2816, 128 rows: 28.4 -> 22.6 us
   // for the whole call.  At ranks 64 and 128 the tcgen05 shrink is the faster one from 256 rows on, with or without overlap.)
   RowsShape shape;
-  const bool few = h.n_rows <= (L->rank <= 32 ? 512 : 256) && rows_shape(ctx, h.n_rows, L->d_out, L->d_in, shape);
+  const bool few = h.n_rows <= (L->rank <= 32 ? 512 : 256) && rows_shape(ctx, h.n_rows, L->d_out, L->d_in, lowrank_columns(h.fwd, L->rank), shape) &&
+                   shrink_few_fits(ctx, L->rank, L->d_in, h.fwd.n_items());
   const bool tc_shrink = !few && ctx->shrink_path == 0 && ctx->drop.thr == 0 && !h.fwd.tcb_row0.empty() &&
                          (L->rank >= kTcShrinkMinRank || ctx->grad_mode == 2) && shrink_tc_fits(ctx, h.fwd, h.n_rows, L->d_in, L->rank);
   if (tc_shrink) {
@@ -1754,7 +1800,8 @@ mlora_status_t mlora_backward(mlora_ctx* ctx, const mlora_layer_t* L, const mlor
   // Whole backward calls with it / with the others, us: 4096 -> 4096 rank 16, 64 rows 27.0 / 28.5; 2560 -> 3968 rank 128,
   // 128 rows 38.6 / 39.9; 2816 -> 10880 rank 16, 64 rows 38.5 / 36.6; 2560 -> 3968 rank 128, 320 rows 53.0 / 49.9)
   RowsShape shape;
-  const bool few = h.ft_rows <= 256 && L->d_out <= 6144 && rows_shape(ctx, h.ft_rows, L->d_in, L->d_out, shape);
+  const bool few = h.ft_rows <= 256 && L->d_out <= 6144 && rows_shape(ctx, h.ft_rows, L->d_in, L->d_out, dropping ? 0 : lowrank_columns(h.bwd, L->rank), shape) &&
+                   shrink_few_fits(ctx, L->rank, L->d_out, h.bwd.n_items());
   const bool tc_v = !few && ctx->shrink_path == 0 && (L->rank >= kTcShrinkMinRank || ctx->grad_mode == 2) &&
                     shrink_tc_fits(ctx, h.bwd, h.ft_rows, L->d_out, L->rank);
   if (tc_v) {

@@ -109,3 +109,26 @@ def test_fp32_tiles_of_eight_rows(sess, rows, d_in, d_out, rank):
     """The fp32 product at row, column and contraction remainders of its 8 x 32 tiles and 32-deep blocks."""
     w = synth.random_workload(1500 + rows, d_in, d_out, rank, 3, rows, dtype="f32", max_seg=max(2, rows // 2), p_finetune=0.5)
     run_and_check(sess, w, synth.make_tensors(w))
+
+
+# (rows, adapters, rank, d_in, d_out, launches of the shrink, of a reduction): 4096 -> 4096 with 256 adapters is 128 low-rank K-blocks
+# in two slices of the few-row GEMM, the two-SM kernel runs them in four and adds these up (64 us against 75); 64 adapters of
+# four rows at rank 128 leave the few-row shrink no CTAs along K, the tcgen05 shrink and its finish kernel take them (52 us
+# against 110 for the call); the same rows of four adapters stay on the few-row kernels
+@pytest.mark.parametrize("rows,adapters,rank,d_in,d_out,shrinks,reductions", [
+    (256, 256, 32, 4096, 4096, 1, 1), (256, 64, 128, 8192, 1024, 2, 0), (256, 4, 128, 4096, 1024, 1, 0), (256, 4, 32, 4096, 4096, 1, 0)])
+def test_batches_of_many_adapters_leave_the_few_row_kernels(sess, rows, adapters, rank, d_in, d_out, shrinks, reductions):
+    n = rows // adapters
+    segs = synth.segments_array([(i * n, n, i, 0) for i in range(adapters)])
+    t = {"X": np.zeros((rows, d_in)), "W": np.zeros((d_in, d_out)), "A_all": np.zeros((adapters, rank, d_in)),
+         "B_all": np.zeros((adapters, rank, d_out)), "scale": np.ones(adapters)}
+    run = LayerRun(sess, "bf16", t, segs, rows)
+    mb.mlora_profile_enable(sess.ctx, 8)
+    try:
+        run.forward()
+        kinds = list(mb.mlora_profile_collect(sess.ctx)[0])
+        assert run.status() == mb.MLORA_OK
+        assert (kinds.count(0), kinds.count(6)) == (shrinks, reductions)
+    finally:
+        mb.mlora_profile_enable(sess.ctx, 0)
+        run.close()
