@@ -45,7 +45,6 @@ struct Args {
   int32_t R;                    // rank
   int32_t lora;                 // 0: base product only
   int32_t early;                // 1: weight and input rows may be read before the dependency wait
-  const __nv_bfloat16* L_all;   // stacked adapter matrices [adapters R, N]
   const int32_t* tile_grp_off;  // groups of each 256-row tile of the batch, and their adapters
   const int32_t* grp_adapter;
   const int32_t* tile_cols;     // plans made with per-adapter ranks (else null): columns of a tile's low-rank operand, first
@@ -297,16 +296,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
       lora_info[t] = !args.tile_cols ? gi * args.R : (gi < n_grp ? args.grp_col[g + gi] : (args.lora ? args.tile_cols[mt] : 0));
     }
     if (t == 2) lora_info[2] = g;
-    asm volatile("bar.sync 2, 128;" ::: "memory");
     asm volatile("bar.arrive 1, 160;\n\tbar.arrive 3, 160;\n\tbar.arrive 4, 160;" ::: "memory");
-    lora_range();
-    // The adapters' rows of this tile are 128-byte pieces all over memory: on their way to the L2 while the main blocks
-    // stream, so that the low-rank blocks behind them do not wait for memory one after the other.
-    for (int i = col_begin + t; i < col_end; i += 128) {
-      const __nv_bfloat16* p = args.L_all + (size_t)(box_row[i / box] + i % box) * args.N + n0;
-      ptx::prefetch_l2(p);
-      if (n0 + 64 < args.N) ptx::prefetch_l2(p + 64);
-    }
     // The MMAs of the low-rank blocks wait for the launch before, so its time must not count against the limit of the wait
     // here.  And no CTA stores or ends before that launch has ended: what follows in the stream may rely on that.
     ptx::grid_dependency_wait();

@@ -1073,7 +1073,6 @@ mlora_status_t launch_gemm_rows(mlora_ctx* ctx, const mlora_layer_t* L, const Ro
   a.M = M; a.N = N; a.K = K; a.R = R; a.nb = nb;
   a.lora = lora && !hs.grp2_adapter.empty() ? 1 : 0;
   a.early = early ? 1 : 0;
-  a.L_all = (const __nv_bfloat16*)L_all;
   a.tile_grp_off = ds.tile2_grp_off; a.grp_adapter = ds.grp2_adapter;
   a.tile_cols = ranked ? ds.tile2_cols : nullptr; a.grp_col = ds.grp2_col; a.tile_piece_off = ds.tile2_piece_off; a.piece_src = ranked ? ds.piece_src : nullptr;
   a.Out = (__nv_bfloat16*)Out; a.ld_out = ld_out; a.status = ctx->status_dev;
