@@ -9,6 +9,7 @@ from paper_2607_28848_b200 import binding as mb
 from paper_2607_28848_b200 import synth
 from paper_2607_28848_b200.runner import LayerRun, Session
 from test_gpu_parity import TOL, assert_close, run_and_check
+from test_gpu_variants import check_dropout
 
 pytestmark = pytest.mark.gpu
 
@@ -109,6 +110,33 @@ def test_fp32_tiles_of_eight_rows(sess, rows, d_in, d_out, rank):
     """The fp32 product at row, column and contraction remainders of its 8 x 32 tiles and 32-deep blocks."""
     w = synth.random_workload(1500 + rows, d_in, d_out, rank, 3, rows, dtype="f32", max_seg=max(2, rows // 2), p_finetune=0.5)
     run_and_check(sess, w, synth.make_tensors(w))
+
+
+@pytest.mark.parametrize("save_x", [True, False])
+@pytest.mark.parametrize("rank", [8, 16, 32, 64, 128])
+@pytest.mark.parametrize("rows", [17, 130, 250])
+def test_dropout(sess, rows, rank, save_x):
+    """The few-row shrink with the dropout mask: above rank 32 several CTAs share a row, each masks it and one saves it.  Saved
+    behind rows of an earlier step; without x_save the forward gives the same Y and u_save."""
+    w = synth.random_workload(1600 + rows + rank, 1088, 448, rank, 4, rows, max_seg=max(2, rows // 3), p_finetune=0.7)
+    t = synth.make_tensors(w)
+    p, seed, base = 0.2, 2 ** 33 + rows, 7
+    if save_x:
+        check_dropout(sess, w, t, p, seed, base=base, cap=base + w.ft_rows + 5)
+        return
+    outs = []
+    mb.mlora_set_dropout(sess.ctx, p, seed)
+    try:
+        for keep in (True, False):
+            run = LayerRun(sess, w.dtype, t, w.segments, w.n_rows, save_row_base=base, save_x=keep)
+            run.forward()
+            assert run.status() == mb.MLORA_OK
+            outs.append((run.host(run.Y), run.host(run.u_save)))
+            run.close()
+    finally:
+        mb.mlora_set_dropout(sess.ctx, 0.0, 0)
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b)
 
 
 # (rows, adapters, rank, d_in, d_out, launches of the shrink, of a reduction): 4096 -> 4096 with 256 adapters is 128 low-rank K-blocks

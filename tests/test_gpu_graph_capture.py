@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("case", ["mixed", "long_k_split", "dropout", "one_finetune_adapter", "rank_128", "uneven_tiles"])
 def test_graph_replay_matches_eager_on_new_inputs(case):
     with Session(0) as sess:
-        if case == "long_k_split":      # few output tiles and K = 8192: the K-split GEMM and its reduction kernel
+        if case == "long_k_split":      # few output tiles and K = 8192: the few-row GEMM in eight K slices
             w = synth.random_workload(62, 8192, 256, 16, 3, 200, max_seg=80, p_finetune=0.5)
         elif case == "one_finetune_adapter":   # gradient groups split over rows: partial sums and arrival counters inside the graph
             segs = synth.segments_array([(0, 60, 2, 0), (60, 900, 0, 1), (960, 40, 1, 0)])

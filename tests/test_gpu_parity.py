@@ -96,14 +96,15 @@ def test_rank_sweep(sess, rank):
 
 @pytest.mark.parametrize("rank", [8, 16, 128])
 def test_no_split_k(sess, rank):
-    """The two-SM kernel without K slices on a small problem (kernel variant 4); the default splits it."""
+    """The two-SM kernel without K slices on a small problem (kernel variant 4); the default takes the few-row kernels."""
     w = synth.random_workload(10 + rank, 320, 448, rank, 7, 300, max_seg=90)
     run_and_check(sess, w, synth.make_tensors(w), path=4)
 
 
 @pytest.mark.parametrize("k", [8192, 8192 + 64 * 37, 16384])
 def test_split_k_slices(sess, k):
-    """Long contractions with few output tiles: 4 to 8 K slices (also a K that the slices do not divide evenly)."""
+    """Long contractions with few output tiles: eight K slices of the few-row GEMM (also a K that they do not divide evenly);
+    tests/test_gpu_paths.py has products that the two-SM kernel cuts into slices."""
     segs = synth.segments_array([(0, 100, 0, 0), (100, 60, 1, 1), (160, 30, 2, 0), (190, 64, 0, 1)])
     w = synth.Workload("split_k", k, 256, 16, 3, "bf16", 254, segs, seed=k)
     run_and_check(sess, w, synth.make_tensors(w), blocked=True)
@@ -193,8 +194,9 @@ def test_row_tiles_of_unequal_cost_get_balanced_unit_lists(sess, rank):
 @pytest.mark.parametrize("d_in,d_out", [(64, 128), (128, 64), (320, 448), (192, 320)])
 def test_output_width_not_a_multiple_of_the_column_tile(sess, path, d_in, d_out):
     """Output widths that leave 1, 2 or 3 of the four 64-column chunks of the last column tile:
-    the epilogue's two staging buffers alternate per chunk whether or not the chunk is stored, so
-    a chunk past the edge must not overwrite a buffer whose store is still in flight.  Repeated on
+    the two-SM and one-SM epilogues' two staging buffers alternate per chunk whether or not the chunk is stored, so
+    a chunk past the edge must not overwrite a buffer whose store is still in flight (path 0 takes the few-row kernels
+    here; tests/test_gpu_paths.py runs the two-SM epilogue).  Repeated on
     a warm context, since a slip here is a race (it showed as zeros in the last rows of a 32-row box)."""
     w = synth.random_workload(900 + d_in + d_out, d_in, d_out, 32, 20, 183, max_seg=60, p_finetune=0.9)
     t = synth.make_tensors(w)
