@@ -233,9 +233,17 @@ def table_sweep(args):
 def table_smallbatch(args):
     if not torch.cuda.is_available():
         raise RuntimeError("small-batch timings need the CUDA path: no GPU visible")
-    lines = ["| projection | rows (inference + fine-tune) | forward µs: no split / default | backward µs: no split / default |",
+    # kernel variant 4: the two-SM GEMM without K slices, no few-row kernels; the default takes the few-row kernels, or the
+    # two-SM GEMM with or without K slices (marked where its reduction kernel runs)
+    lines = ["| projection | rows (inference + fine-tune) | forward µs: variant 4 / default | backward µs: variant 4 / default |",
              "|---|---|---|---|"]
     with Session(0) as sess:
+        def sliced(fn):
+            mb.mlora_profile_enable(sess.ctx, 16)
+            fn()
+            kinds, _ = mb.mlora_profile_collect(sess.ctx, 16)
+            mb.mlora_profile_enable(sess.ctx, 0)
+            return " (K slices)" if KIND_REDUCE in kinds else ""
         for t_ft in (256, 512):
             for d_in, d_out in ((4096, 4096), (4096, 14336), (14336, 4096)):
                 segs = synth.segments_array([(0, 256, 1, 0), (256, t_ft, 0, 1)])
@@ -246,10 +254,11 @@ def table_smallbatch(args):
                     mb.mlora_set_gemm_path(sess.ctx, path)
                     res[path] = (timeit(run.forward), timeit(run.backward))
                 mb.mlora_set_gemm_path(sess.ctx, 0)
+                how = (sliced(run.forward), sliced(run.backward))
                 if run.status() != mb.MLORA_OK:
                     raise RuntimeError("device status non-zero")
                 run.close()
-                lines.append(f"| {d_in} → {d_out} | 256 + {t_ft} | {res[4][0]:.1f} / {res[0][0]:.1f} | {res[4][1]:.1f} / {res[0][1]:.1f} |")
+                lines.append(f"| {d_in} → {d_out} | 256 + {t_ft} | {res[4][0]:.1f} / {res[0][0]:.1f}{how[0]} | {res[4][1]:.1f} / {res[0][1]:.1f}{how[1]} |")
         # decode-sized forward calls: back to back (launch overlap on), and each kernel with its own event pair
         lines += ["", "| projection | decode rows | µs per forward call back to back | weight read once at the measured copy bandwidth | shrink / GEMM / reduction (event pairs) |",
                   "|---|---|---|---|---|"]

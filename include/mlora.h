@@ -326,13 +326,17 @@ int32_t mlora_profile_collect(mlora_ctx* ctx, int32_t* kinds, float* ms, int32_t
 /* Selects kernel variants for MLORA_BF16 layers: 0 = defaults (two-SM tcgen05 tensor-core GEMM; rank <= 16:
  * streaming mma.sync shrink and gradient kernels; rank 32, 64 and 128: the tcgen05 shrink with its finish
  * kernel for U = X A^T and V = s dY B^T wherever the rows come in runs of eight (rank 128: four) or more
- * per adapter on average, and the tcgen05 gradient kernel); 1 = the plain CUDA-core kernels for every step (a slow
- * cross-check used by the tests); 2 = defaults, but the per-item mma.sync shrink and gradient kernels
- * for every rank; 3 = defaults, but the one-SM tensor-core GEMM;
- * 4 = defaults, but the two-SM GEMM never splits K (by default a product with too few output
+ * per adapter on average, and the tcgen05 gradient kernel.  A product of few rows - its tiles of 128 output
+ * columns and up to 128 rows number at most one per SM, and neither its contraction nor its adapters are too
+ * many for that split - takes the few-row GEMM instead, whose K slices are summed inside a cluster; up to 512
+ * rows (256 above rank 32; 256 in the backward) the few-row shrink goes with it where each adapter's rows are
+ * few enough too); 1 = the plain CUDA-core kernels for every step (a slow
+ * cross-check used by the tests).  2 to 6 never take the few-row kernels: 2 = the per-item mma.sync shrink and
+ * gradient kernels for every rank; 3 = the one-SM tensor-core GEMM;
+ * 4 = the two-SM GEMM never splits K (by default a product with too few output
  * tiles for the SMs is cut into K slices whose fp32 partials a small kernel adds up);
- * 5 = defaults, but both gradients on the mma.sync kernels for every rank;
- * 6 = defaults, but every rank-r product on the tcgen05 kernels for every rank: U, V and both gradients
+ * 5 = both gradients on the mma.sync kernels for every rank;
+ * 6 = every rank-r product on the tcgen05 kernels for every rank: U, V and both gradients
  * (with dropout on, everything stays on the mma.sync kernels);
  * 7 = defaults, but the two-SM GEMM always deals its tiles out round robin (by default a batch whose
  * 256-row tiles differ much in their number of adapter groups gets, per shape it is used with, a list
