@@ -194,6 +194,14 @@ mlora_status_t mlora_mixed_forward(mlora_ctx* ctx, const mlora_layer_t* layer, c
                                    int64_t save_row_base, int64_t save_capacity_rows,
                                    void* cuda_stream);
 
+/* What mlora_mixed_forward writes to x_save and u_save for the plan's fine-tuning rows - the same bits - without its output:
+ * the end of a recompute pass whose last product nobody reads (paper, Section 3.2: the backward recomputes the layer from its
+ * saved input).  Arguments and errors as there. */
+mlora_status_t mlora_forward_save(mlora_ctx* ctx, const mlora_layer_t* layer, const mlora_plan* plan,
+                                  const void* X, int64_t ldx, void* x_save, float* u_save,
+                                  int64_t save_row_base, int64_t save_capacity_rows,
+                                  void* cuda_stream);
+
 /* ---- backward --------------------------------------------------------------------------*/
 
 /* LoRA backward for the plan's fine-tuning rows (paper, Section 3.2 "Backward subprocess":

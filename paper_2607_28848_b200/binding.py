@@ -26,7 +26,7 @@ EXPORTS = (
     "mlora_backward", "mlora_poll_status", "mlora_status_string", "mlora_launch_count", "mlora_set_gemm_path",
     "mlora_plan_create_ranked", "mlora_plan_create_ranked_async", "mlora_plan_lowrank_columns", "mlora_profile_enable", "mlora_profile_collect", "mlora_forward_noalloc", "mlora_adamw_update",
     "mlora_set_cancel_flag", "mlora_set_dropout", "mlora_plan_create_async", "mlora_plan_release",
-    "mlora_selftest_timeout",
+    "mlora_selftest_timeout", "mlora_forward_save",
 )
 MLORA_NOALLOC_MAX_ROWS = 512
 
@@ -99,6 +99,8 @@ def load_library(build_if_missing: bool = True) -> ctypes.CDLL:
     lib.mlora_plan_describe.restype = ctypes.c_int
     lib.mlora_mixed_forward.argtypes = [vp, P(mlora_layer_t), vp, vp, i64, vp, i64, vp, vp, i64, i64, vp]
     lib.mlora_mixed_forward.restype = ctypes.c_int
+    lib.mlora_forward_save.argtypes = [vp, P(mlora_layer_t), vp, vp, i64, vp, vp, i64, i64, vp]
+    lib.mlora_forward_save.restype = ctypes.c_int
     lib.mlora_backward.argtypes = [vp, P(mlora_layer_t), vp, vp, i64, vp, vp, vp, vp, vp, i64, i32, vp]
     lib.mlora_backward.restype = ctypes.c_int
     lib.mlora_poll_status.argtypes = [vp, vp]
@@ -279,6 +281,17 @@ def mlora_mixed_forward(ctx, layer: mlora_layer_t, plan, X, Y, x_save, u_save, s
         _ptr(Y), Y.stride(0) if Y is not None else 0, _ptr(x_save), _ptr(u_save),
         int(save_row_base), int(save_capacity_rows), _stream_ptr(stream))
     _check(st, "mlora_mixed_forward")
+
+
+def mlora_forward_save(ctx, layer: mlora_layer_t, plan, X, x_save, u_save, save_row_base: int = 0,
+                       save_capacity_rows: Optional[int] = None, stream=None) -> None:
+    """Queue what `mlora_mixed_forward` saves for the fine-tuning rows (x_save, u_save) without its output."""
+    if save_capacity_rows is None:
+        save_capacity_rows = 0 if u_save is None else int(u_save.shape[0])
+    st = load_library().mlora_forward_save(
+        ctx, ctypes.byref(layer), plan, _ptr(X), X.stride(0) if X is not None else 0, _ptr(x_save), _ptr(u_save),
+        int(save_row_base), int(save_capacity_rows), _stream_ptr(stream))
+    _check(st, "mlora_forward_save")
 
 
 def mlora_backward(ctx, layer: mlora_layer_t, plan, dY, x_save, u_save, dA, dB, dX, accumulate: bool = False,

@@ -1253,6 +1253,56 @@ mlora_status_t backward_simt(mlora_ctx* ctx, const mlora_layer_t* L, const mlora
   return s;
 }
 
+// What a forward asks of its arguments but for the output (MLORA_OK with no rows: nothing behind the plan was looked at).
+mlora_status_t check_forward(const mlora_ctx* ctx, const mlora_layer_t* L, const mlora_plan* p, const void* X, int64_t ldx, const float* u_save,
+                             int64_t save_row_base, int64_t save_capacity_rows) {
+  if (!ctx || !p || p->ctx != ctx || !p->blob) return MLORA_ERR_INVALID_ARG;
+  const mlora_status_t s = check_layer(L);
+  if (s != MLORA_OK) return s;
+  const HostPlan& h = p->h;
+  if (h.n_adapters > L->n_adapters) return MLORA_ERR_ADAPTER_ID;
+  if (h.n_rows == 0) return MLORA_OK;
+  if (!X || ldx < L->d_in) return MLORA_ERR_INVALID_ARG;
+  if (save_row_base < 0 || save_capacity_rows < 0) return MLORA_ERR_INVALID_ARG;
+  if (h.ft_rows > 0) {
+    if (save_row_base + h.ft_rows > save_capacity_rows) return MLORA_ERR_SAVE_CAPACITY;
+    if (!u_save) return MLORA_ERR_INVALID_ARG;
+  }
+  return h.n_rows > ctx->ws_rows || !ranked_plan_fits(h, L) ? MLORA_ERR_INVALID_ARG : MLORA_OK;
+}
+
+// The rank-r product of a forward with its activation save, bf16 layers; `product`: the GEMM's low-rank operand as well.
+mlora_status_t forward_shrink(mlora_ctx* ctx, const mlora_layer_t* L, const mlora_plan* p, const void* X, int64_t ldx, void* x_save,
+                              float* u_save, int64_t save_row_base, int64_t save_capacity_rows, bool product, cudaStream_t st) {
+  const HostPlan& h = p->h;
+  ShrinkArgs sa;
+  sa.In = (const __nv_bfloat16*)X; sa.ld_in = ldx; sa.D = L->d_in;
+  sa.P_all = (const __nv_bfloat16*)L->A_all; sa.scale = nullptr; sa.Out = ctx->ws_p;
+  sa.item_rows = p->fwd.item_rows; sa.item_start = p->fwd.item_start; sa.item_nrows = p->fwd.item_nrows;
+  sa.item_adapter = p->fwd.item_adapter; sa.item_save = p->fwd.item_save;
+  sa.pbd = PbdArgs{ctx->gemm_pairs && product ? ctx->ws_pbd : nullptr, p->fwd.row_grp2, p->fwd.tile2_grp_off, L->scale,
+                   p->fwd.zero_rows2, (int32_t)h.fwd.zero_rows2.size()};
+  set_ranked(sa.pbd, p->fwd);
+  sa.x_save = (__nv_bfloat16*)x_save; sa.u_save = u_save; sa.save_base = save_row_base;
+  sa.save_cap = save_capacity_rows;
+  // rank >= kTcShrinkMinRank (every rank under kernel variant 6): the tcgen05 shrink and its finish kernel
+  // (a batch of few rows: the latency-bound shrink that its GEMM overlaps with; 10880 -> 2816, 128 rows: 28.4 -> 22.6 us
+  // for the whole call.  At ranks 64 and 128 the tcgen05 shrink is the faster one from 256 rows on, with or without overlap.)
+  RowsShape shape;
+  const bool few = h.n_rows <= (L->rank <= 32 ? 512 : 256) && rows_shape(ctx, h.n_rows, L->d_out, L->d_in, lowrank_columns(h.fwd, L->rank), shape) &&
+                   shrink_few_fits(ctx, L->rank, L->d_in, h.fwd.n_items());
+  const bool tc_shrink = !few && ctx->shrink_path == 0 && ctx->drop.thr == 0 && !h.fwd.tcb_row0.empty() &&
+                         (L->rank >= kTcShrinkMinRank || ctx->grad_mode == 2) && shrink_tc_fits(ctx, h.fwd, h.n_rows, L->d_in, L->rank);
+  if (tc_shrink) {
+    stc::FinArgs fa = {};
+    fa.scale = nullptr; fa.Out = ctx->ws_p; fa.pbd = sa.pbd;
+    fa.row_save = h.ft_rows > 0 ? p->fwd.row_save : nullptr; fa.u_save = u_save;
+    fa.X = (const __nv_bfloat16*)X; fa.ldx = ldx; fa.x_save = (__nv_bfloat16*)x_save; fa.save_base = save_row_base; fa.D = L->d_in;
+    return launch_shrink_tc_any(ctx, L->rank, h.fwd, p->fwd, X, ldx, h.n_rows, L->d_in, L->A_all, L->n_adapters, fa, st);
+  }
+  return launch_shrink(ctx, L->rank, sa, h.fwd.n_items(), p->fwd.item_desc, h.n_rows, L->n_adapters, few, st);
+}
+
 }  // namespace
 
 // ---- allocation-free forward ------------------------------------------------------------------
@@ -1706,19 +1756,11 @@ mlora_status_t mlora_plan_describe(const mlora_plan* p, int32_t* seg_save_offset
 mlora_status_t mlora_mixed_forward(mlora_ctx* ctx, const mlora_layer_t* L, const mlora_plan* p, const void* X,
                                    int64_t ldx, void* Y, int64_t ldy, void* x_save, float* u_save,
                                    int64_t save_row_base, int64_t save_capacity_rows, void* cuda_stream) {
-  if (!ctx || !p || p->ctx != ctx || !p->blob) return MLORA_ERR_INVALID_ARG;
-  mlora_status_t s = check_layer(L);
+  mlora_status_t s = check_forward(ctx, L, p, X, ldx, u_save, save_row_base, save_capacity_rows);
   if (s != MLORA_OK) return s;
   const HostPlan& h = p->h;
-  if (h.n_adapters > L->n_adapters) return MLORA_ERR_ADAPTER_ID;
   if (h.n_rows == 0) return MLORA_OK;
-  if (!X || !Y || ldx < L->d_in || ldy < L->d_out) return MLORA_ERR_INVALID_ARG;
-  if (save_row_base < 0 || save_capacity_rows < 0) return MLORA_ERR_INVALID_ARG;
-  if (h.ft_rows > 0) {
-    if (save_row_base + h.ft_rows > save_capacity_rows) return MLORA_ERR_SAVE_CAPACITY;
-    if (!u_save) return MLORA_ERR_INVALID_ARG;
-  }
-  if (h.n_rows > ctx->ws_rows || !ranked_plan_fits(h, L)) return MLORA_ERR_INVALID_ARG;
+  if (!Y || ldy < L->d_out) return MLORA_ERR_INVALID_ARG;
   // the tensor maps are encoded through the driver API, which needs this device's context current on the
   // calling thread (a framework's worker threads do not always have one)
   if (cudaSetDevice(ctx->device) != cudaSuccess) return MLORA_ERR_CUDA;
@@ -1730,36 +1772,26 @@ mlora_status_t mlora_mixed_forward(mlora_ctx* ctx, const mlora_layer_t* L, const
     return forward_simt<__nv_bfloat16>(ctx, L, p, X, ldx, Y, ldy, x_save, u_save, save_row_base, st);
 
   if (ctx->drop.thr != 0 && h.ft_rows > 0 && ctx->shrink_path != 0 && L->rank <= 64) return MLORA_ERR_UNSUPPORTED;
-  ShrinkArgs sa;
-  sa.In = (const __nv_bfloat16*)X; sa.ld_in = ldx; sa.D = L->d_in;
-  sa.P_all = (const __nv_bfloat16*)L->A_all; sa.scale = nullptr; sa.Out = ctx->ws_p;
-  sa.item_rows = p->fwd.item_rows; sa.item_start = p->fwd.item_start; sa.item_nrows = p->fwd.item_nrows;
-  sa.item_adapter = p->fwd.item_adapter; sa.item_save = p->fwd.item_save;
-  sa.pbd = PbdArgs{ctx->gemm_pairs ? ctx->ws_pbd : nullptr, p->fwd.row_grp2, p->fwd.tile2_grp_off, L->scale,
-                   p->fwd.zero_rows2, (int32_t)h.fwd.zero_rows2.size()};
-  set_ranked(sa.pbd, p->fwd);
-  sa.x_save = (__nv_bfloat16*)x_save; sa.u_save = u_save; sa.save_base = save_row_base;
-  sa.save_cap = save_capacity_rows;
-  // rank >= kTcShrinkMinRank (every rank under kernel variant 6): the tcgen05 shrink and its finish kernel
-  // (a batch of few rows: the latency-bound shrink that its GEMM overlaps with; 10880 -> 2816, 128 rows: 28.4 -> 22.6 us
-  // for the whole call.  At ranks 64 and 128 the tcgen05 shrink is the faster one from 256 rows on, with or without overlap.)
-  RowsShape shape;
-  const bool few = h.n_rows <= (L->rank <= 32 ? 512 : 256) && rows_shape(ctx, h.n_rows, L->d_out, L->d_in, lowrank_columns(h.fwd, L->rank), shape) &&
-                   shrink_few_fits(ctx, L->rank, L->d_in, h.fwd.n_items());
-  const bool tc_shrink = !few && ctx->shrink_path == 0 && ctx->drop.thr == 0 && !h.fwd.tcb_row0.empty() &&
-                         (L->rank >= kTcShrinkMinRank || ctx->grad_mode == 2) && shrink_tc_fits(ctx, h.fwd, h.n_rows, L->d_in, L->rank);
-  if (tc_shrink) {
-    stc::FinArgs fa = {};
-    fa.scale = nullptr; fa.Out = ctx->ws_p; fa.pbd = sa.pbd;
-    fa.row_save = h.ft_rows > 0 ? p->fwd.row_save : nullptr; fa.u_save = u_save;
-    fa.X = (const __nv_bfloat16*)X; fa.ldx = ldx; fa.x_save = (__nv_bfloat16*)x_save; fa.save_base = save_row_base; fa.D = L->d_in;
-    s = launch_shrink_tc_any(ctx, L->rank, h.fwd, p->fwd, X, ldx, h.n_rows, L->d_in, L->A_all, L->n_adapters, fa, st);
-  } else {
-    s = launch_shrink(ctx, L->rank, sa, h.fwd.n_items(), p->fwd.item_desc, h.n_rows, L->n_adapters, few, st);
-  }
-  if (s != MLORA_OK) return s;
+  if ((s = forward_shrink(ctx, L, p, X, ldx, x_save, u_save, save_row_base, save_capacity_rows, true, st)) != MLORA_OK) return s;
   return gemm_bf16<false>(ctx, L, h.fwd, p->fwd, X, ldx, Y, ldy, L->B_all, ctx->ws_p, L->scale, h.n_rows, L->d_out,
                           L->d_in, st, h.fwd.n_items() > 0);
+}
+
+mlora_status_t mlora_forward_save(mlora_ctx* ctx, const mlora_layer_t* L, const mlora_plan* p, const void* X, int64_t ldx, void* x_save,
+                                  float* u_save, int64_t save_row_base, int64_t save_capacity_rows, void* cuda_stream) {
+  const mlora_status_t s = check_forward(ctx, L, p, X, ldx, u_save, save_row_base, save_capacity_rows);
+  if (s != MLORA_OK || p->h.n_rows == 0) return s;
+  if (cudaSetDevice(ctx->device) != cudaSuccess) return MLORA_ERR_CUDA;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
+  if (L->dtype == MLORA_F32)
+    return simt_shrink<float>(ctx, (const float*)X, ldx, L->d_in, L->rank, (const float*)L->A_all, nullptr, p->fwd, ctx->ws_p, (float*)x_save, u_save,
+                              save_row_base, p->h.n_rows, L->n_adapters, ctx->drop, st);
+  if (ldx % 8 || !aligned16(X) || (x_save && !aligned16(x_save))) return MLORA_ERR_UNSUPPORTED;
+  if (ctx->gemm_path == 1)
+    return simt_shrink<__nv_bfloat16>(ctx, (const __nv_bfloat16*)X, ldx, L->d_in, L->rank, (const __nv_bfloat16*)L->A_all, nullptr, p->fwd, ctx->ws_p,
+                                      (__nv_bfloat16*)x_save, u_save, save_row_base, p->h.n_rows, L->n_adapters, ctx->drop, st);
+  if (ctx->drop.thr != 0 && p->h.ft_rows > 0 && ctx->shrink_path != 0 && L->rank <= 64) return MLORA_ERR_UNSUPPORTED;
+  return forward_shrink(ctx, L, p, X, ldx, x_save, u_save, save_row_base, save_capacity_rows, false, st);
 }
 
 mlora_status_t mlora_backward(mlora_ctx* ctx, const mlora_layer_t* L, const mlora_plan* p, const void* dY, int64_t lddy,

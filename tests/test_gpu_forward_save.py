@@ -1,0 +1,43 @@
+"""The activation save without the output: the same bits as the forward writes, on every kernel that it can take."""
+import pytest
+import torch
+
+from paper_2607_28848_b200 import binding as mb
+from paper_2607_28848_b200 import synth
+from paper_2607_28848_b200.runner import LayerRun, Session
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sess():
+    s = Session(0)
+    yield s
+    s.close()
+
+
+# few-row, streaming and tcgen05 shrinks, with and without a mask, a saved base, the fp32 kernels
+@pytest.mark.parametrize("dtype,rows,d_in,d_out,rank,dropout", [
+    ("bf16", 70, 1024, 320, 16, 0.0), ("bf16", 70, 1024, 320, 16, 0.1), ("bf16", 900, 1024, 4096, 16, 0.0), ("bf16", 900, 576, 4096, 64, 0.0),
+    ("bf16", 900, 576, 4096, 128, 0.1), ("f32", 60, 96, 64, 8, 0.0), ("f32", 60, 96, 64, 8, 0.1)])
+def test_saves_what_the_forward_saves(sess, dtype, rows, d_in, d_out, rank, dropout):
+    w = synth.random_workload(1700 + rows + rank, d_in, d_out, rank, 5, rows, dtype=dtype, max_seg=max(2, rows // 3), p_finetune=0.6)
+    run = LayerRun(sess, w.dtype, synth.make_tensors(w), w.segments, w.n_rows, save_row_base=3)
+    try:
+        mb.mlora_set_dropout(sess.ctx, dropout, 11)
+        run.forward()
+        want = run.x_save.clone(), run.u_save.clone()
+        run.x_save[3:].zero_()
+        run.u_save[3:].zero_()
+        Y = run.Y.clone()
+        mb.mlora_forward_save(sess.ctx, run.layer, run.plan, run.X, run.x_save, run.u_save, 3)
+        assert run.status() == mb.MLORA_OK
+        assert torch.equal(run.x_save, want[0]) and torch.equal(run.u_save, want[1]) and torch.equal(run.Y, Y)
+        u = run.u_save.clone().zero_()
+        mb.mlora_forward_save(sess.ctx, run.layer, run.plan, run.X, None, u, 3)
+        assert torch.equal(u[3:3 + w.ft_rows], want[1][3:3 + w.ft_rows])
+        with pytest.raises(mb.MloraError):
+            mb.mlora_forward_save(sess.ctx, run.layer, run.plan, run.X, None, u, u.shape[0] - w.ft_rows + 1)
+    finally:
+        mb.mlora_set_dropout(sess.ctx, 0.0, 0)
+        run.close()
