@@ -161,7 +161,7 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
   uint32_t* tmem_ptr_smem = reinterpret_cast<uint32_t*>(smem_gen + (sMisc - smem_base));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + (sMisc - smem_base) + 8);
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = ptx::warp_uniform(threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   const uint32_t rank = ptx::cluster_ctarank();     // 0: leader
   const bool leader = rank == 0;
@@ -191,7 +191,7 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
   __syncthreads();
   ptx::cluster_sync_all();                           // the peer's barriers exist from here on
   ptx::tc_fence_after();
-  const uint32_t tmem_base = *tmem_ptr_smem;
+  const uint32_t tmem_base = ptx::warp_uniform(*tmem_ptr_smem);
   if (!args.early) ptx::grid_dependency_wait();
   ptx::grid_launch_dependents();
 
@@ -212,7 +212,7 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
 
   if (warp == 0) {
     // ============================ TMA producer (both CTAs) ============================
-    // Lane 0 waits and issues the main loads; the low-rank stages are issued by all lanes, one
+    // One elected lane issues the main loads; the low-rank stages are issued by all lanes, one
     // adapter group per lane, from a copy of the tile's adapter list in shared memory, so that
     // the list costs one memory latency per tile rather than one per group.
     int32_t* ga_smem = reinterpret_cast<int32_t*>(smem_gen + (sMisc - smem_base) + 64);   // 256 entries
@@ -242,19 +242,16 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
       }
       for (int kb = kb_begin; kb < kb_end; ++kb, ++it) {
         const int s = it % S;
-        if (lane == 0) {
-          ok = gemm2_wait(bar_empty(s), ((it / S) & 1) ^ 1, abort_flag, args.status);
-          if (ok) {
-            const uint32_t a = sA0 + s * GEMM2_STAGE_BYTES, b = a + GEMM2_A_BYTES;
-            const uint32_t full = ptx::map_to_cta(bar_full(s), 0);
-            if (leader) ptx::mbar_arrive_expect_tx(bar_full(s), 2 * GEMM2_STAGE_BYTES);
-            ptx::tma2_load_2d(a, &tmIn, kb * GEMM_BK, m0, full);
-            if (W_KMAJOR) ptx::tma2_load_2d(b, &tmW, kb * GEMM_BK, nh, full);          // [N, K]: 128 rows x 64 k
-            else          ptx::tma2_load_3d(b, &tmW, 0, kb * GEMM_BK, nh >> 6, full);  // (64 n, K, N/64): 64 x 64 k x 2
-          }
-        }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        ok = ptx::warp_all(gemm2_wait(bar_empty(s), ((it / S) & 1) ^ 1, abort_flag, args.status));
         if (!ok) break;
+        const uint32_t a = sA0 + s * GEMM2_STAGE_BYTES, b = a + GEMM2_A_BYTES;
+        const uint32_t full = ptx::map_to_cta(bar_full(s), 0);
+        if (ptx::elect_one()) {
+          if (leader) ptx::mbar_arrive_expect_tx(bar_full(s), 2 * GEMM2_STAGE_BYTES);
+          ptx::tma2_load_2d(a, &tmIn, kb * GEMM_BK, m0, full);
+          if (W_KMAJOR) ptx::tma2_load_2d(b, &tmW, kb * GEMM_BK, nh, full);          // [N, K]: 128 rows x 64 k
+          else          ptx::tma2_load_3d(b, &tmW, 0, kb * GEMM_BK, nh >> 6, full);  // (64 n, K, N/64): 64 x 64 k x 2
+        }
       }
       if (!ok) break;
       // The low-rank operand comes from the launch before.  Every role waits for that launch behind the first main loop, low-rank
@@ -319,7 +316,12 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
     __syncwarp();
   } else if (warp == 1) {
     // ============================ MMA issuer (leader only) ============================
-    if (leader && lane == 0) {
+    // The whole warp walks the loop and one elected lane issues, here and in the producer: what a branch of a single lane computes
+    // (descriptors, coordinates, barrier addresses) is not known to be uniform and reaches the uniform registers, where these
+    // instructions take their operands from, one by one.  A K-block took 0.32 us whatever its MMAs needed (0.26 at this width).
+    // Product alone, both sides in turn: 4096 x 4096 x 4096 86.4 -> 80.9 us on zeros, 113 -> 105 on random values under the power
+    // cap, 2560 x 5120 x 13824 282 -> 270, 2048 x 14336 x 4096 199 -> 188, 1600 x 4096 x 4096 46.8 -> 44.6.
+    if (leader) {
       constexpr uint32_t idesc_main = ptx::make_idesc_bf16(GEMM2_BM, GEMM2_BN, false, !W_KMAJOR);
       constexpr uint32_t idesc_lora = ptx::make_idesc_bf16(GEMM2_BM, GEMM2_BN, false, true);
       uint32_t it = 0, lt = 0;
@@ -334,24 +336,25 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
         // columns of the tile's low-rank operand (read here, so that the main loop hides the latency)
         const int lcols = (args.piece_src != nullptr && args.lora_enabled) ? args.tile_cols[mt] : tile_groups(mt) * R;
         const uint32_t buf = lt & 1;
-        if (!(ok = gemm2_wait(bar_tempty(buf), ((lt >> 1) & 1) ^ 1, abort_flag, args.status))) break;
+        if (!(ok = ptx::warp_all(gemm2_wait(bar_tempty(buf), ((lt >> 1) & 1) ^ 1, abort_flag, args.status)))) break;
         ptx::tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * GEMM2_BN;
         uint32_t acc = 0;
         for (int kb = kb_begin; kb < kb_end; ++kb, ++it) {
           const int s = it % S;
-          if (!(ok = gemm2_wait(bar_full(s), (it / S) & 1, abort_flag, args.status))) break;
+          if (!(ok = ptx::warp_all(gemm2_wait(bar_full(s), (it / S) & 1, abort_flag, args.status)))) break;
           ptx::tc_fence_after();
           const uint32_t a = sA0 + s * GEMM2_STAGE_BYTES, b = a + GEMM2_A_BYTES;
           const uint64_t adesc = ptx::make_smem_desc(a, 16, 1024);
           const uint64_t bdesc = W_KMAJOR ? ptx::make_smem_desc(b, 16, 1024) : ptx::make_smem_desc(b, 8192, 1024);
+          if (ptx::elect_one()) {
 #pragma unroll
-          for (int ks = 0; ks < GEMM_BK / 16; ++ks) {
-            ptx::umma2_f16(d_tmem, adesc + (uint64_t)(ks * 2), bdesc + (uint64_t)(W_KMAJOR ? ks * 2 : ks * 128),
-                           idesc_main, acc);
-            acc = 1;
+            for (int ks = 0; ks < GEMM_BK / 16; ++ks)
+              ptx::umma2_f16(d_tmem, adesc + (uint64_t)(ks * 2), bdesc + (uint64_t)(W_KMAJOR ? ks * 2 : ks * 128),
+                             idesc_main, ks == 0 ? acc : 1u);
+            ptx::umma2_commit_both(bar_empty(s));
           }
-          ptx::umma2_commit_both(bar_empty(s));
+          acc = 1;
         }
         if (!ok) break;
         if (args.early && ui == u_begin) ptx::grid_dependency_wait();      // as the producer
@@ -359,21 +362,23 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
         const int lc_begin = (int)((long long)ks * LC / SK), lc_end = (int)((long long)(ks + 1) * LC / SK);
         for (int lc = lc_begin; lc < lc_end; ++lc, ++it) {
           const int s = it % S;
-          if (!(ok = gemm2_wait(bar_full(s), (it / S) & 1, abort_flag, args.status))) break;
+          if (!(ok = ptx::warp_all(gemm2_wait(bar_full(s), (it / S) & 1, abort_flag, args.status)))) break;
           ptx::tc_fence_after();
           const uint32_t a = sA0 + s * GEMM2_STAGE_BYTES, b = a + GEMM2_A_BYTES;
           const uint64_t adesc = ptx::make_smem_desc(a, 16, 1024);
           const uint64_t bdesc = ptx::make_smem_desc(b, 8192, 1024);
           int ksteps = (lcols - lc * 64 + 15) / 16;
           ksteps = ksteps < 4 ? ksteps : 4;
-          for (int ks = 0; ks < ksteps; ++ks) {
-            ptx::umma2_f16(d_tmem, adesc + (uint64_t)(ks * 2), bdesc + (uint64_t)(ks * 128), idesc_lora, acc);
-            acc = 1;
+          if (ptx::elect_one()) {
+#pragma unroll
+            for (int ks = 0; ks < GEMM_BK / 16; ++ks)
+              if (ks < ksteps) ptx::umma2_f16(d_tmem, adesc + (uint64_t)(ks * 2), bdesc + (uint64_t)(ks * 128), idesc_lora, ks == 0 ? acc : 1u);
+            ptx::umma2_commit_both(bar_empty(s));
           }
-          ptx::umma2_commit_both(bar_empty(s));
+          acc = 1;
         }
         if (!ok) break;
-        ptx::umma2_commit_both(bar_tfull(buf));
+        if (ptx::elect_one()) ptx::umma2_commit_both(bar_tfull(buf));
       }
     }
     __syncwarp();

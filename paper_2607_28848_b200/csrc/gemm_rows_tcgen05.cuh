@@ -92,7 +92,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
   auto bar_empty = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
   const uint32_t bar_done = bar0 + 8u * (2 * MAX_STAGES), bar_sums = bar_done + 8u;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = ptx::warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int S = args.stages, SK = args.slices, nb = args.nb;
   const int tile = (int)blockIdx.x / SK, ks = (int)blockIdx.x - tile * SK;
   const int rt = tile / args.col_tiles;
@@ -123,7 +123,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
-  const uint32_t tmem_base = tmem_ptr;
+  const uint32_t tmem_base = ptx::warp_uniform(tmem_ptr);
   if (!args.early) ptx::grid_dependency_wait();
   ptx::grid_launch_dependents();
 
@@ -148,20 +148,16 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
   if (warp == 0) {
     // ============================ TMA producer: weight blocks, then the adapters' rows ============================
     Ring at(S);
-    int ok = 1;
-    if (lane == 0) {
-      for (int kb = kb_begin; kb < kb_end; ++kb, at.next()) {
-        if (!(ok = gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status))) break;
-        const uint32_t w = ring + (uint32_t)at.slot * stage, full = bar_full(at.slot);
+    bool ok = true;
+    for (int kb = kb_begin; kb < kb_end; ++kb, at.next()) {
+      if (!(ok = ptx::warp_all(gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status)))) break;
+      const uint32_t w = ring + (uint32_t)at.slot * stage, full = bar_full(at.slot);
+      if (ptx::elect_one()) {
         ptx::mbar_arrive_expect_tx(full, KW * W_BYTES);
         if (W_KMAJOR) ptx::tma_load_3d(w, &tmW, 0, n0, kb * KW, full);                   // (64 k, N, K/64): KW blocks of 128 rows x 64 k
         else          ptx::tma_load_3d(w, &tmW, 0, kb * KW * GEMM_BK, n0 >> 6, full);    // (64 n, K, N/64): 2 blocks of 64 KW k x 64 n
       }
     }
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    at.slot = __shfl_sync(0xffffffffu, at.slot, 0);
-    at.parity = __shfl_sync(0xffffffffu, at.parity, 0);
-    at.used = __shfl_sync(0xffffffffu, at.used, 0);
     asm volatile("bar.sync 1, 160;" ::: "memory");
     lora_range();
     const int box_begin = col_begin / box, box_end = (col_end + box - 1) / box;
@@ -169,9 +165,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
     for (int lc = col_begin / 64; lc * 64 < col_end && ok; lc += KW, at.next()) {
       // From the second lap on a slot comes free as the MMA warp goes through low-rank blocks, which wait for the launch before.
       if (args.early && fills++ == S) ptx::grid_dependency_wait();
-      if (lane == 0) ok = gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status);
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) break;
+      if (!(ok = ptx::warp_all(gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status)))) break;
       const int j0 = box_begin > lc * per ? box_begin : lc * per, j1 = box_end < (lc + KW) * per ? box_end : (lc + KW) * per;
       const int n = box == 8 ? (j1 - j0 + 1) & ~1 : j1 - j0;     // rank 8: a half-filled MMA step repeats the last group (its operand columns are zero)
       const uint32_t w = ring + (uint32_t)at.slot * stage, full = bar_full(at.slot);
@@ -187,11 +181,11 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
   } else if (warp == 6) {
     // ============================ TMA producer: input rows, then their low-rank operand ============================
     Ring at(S);
-    int ok = 1;
-    if (lane == 0) {
-      for (int kb = kb_begin; kb < kb_end; ++kb, at.next()) {
-        if (!(ok = gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status))) break;
-        const uint32_t x = ring + (uint32_t)at.slot * stage + KW * W_BYTES, full = bar_full(at.slot);
+    bool ok = true;
+    for (int kb = kb_begin; kb < kb_end; ++kb, at.next()) {
+      if (!(ok = ptx::warp_all(gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status)))) break;
+      const uint32_t x = ring + (uint32_t)at.slot * stage + KW * W_BYTES, full = bar_full(at.slot);
+      if (ptx::elect_one()) {
         ptx::mbar_arrive_expect_tx(full, KW * xblk);
         ptx::tma_load_3d(x, &tmIn, 0, m0, kb * KW, full);                          // (64 k, M, K/64): KW blocks of nb rows x 64 k
       }
@@ -199,79 +193,83 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
     __syncwarp();
     asm volatile("bar.sync 3, 160;" ::: "memory");
     lora_range();
-    if (lane == 0) {
-      if (args.early && col_begin < col_end) ptx::grid_dependency_wait();            // the operand comes from the launch before
-      for (int lc = col_begin / 64; lc * 64 < col_end && ok; lc += KW, at.next()) {
-        if (!(ok = gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status))) break;
-        const uint32_t x = ring + (uint32_t)at.slot * stage + KW * W_BYTES, full = bar_full(at.slot);
-        const int n = KW == 1 || (lc + 1) * 64 >= col_end ? 1 : KW;
+    if (args.early && col_begin < col_end) ptx::grid_dependency_wait();              // the operand comes from the launch before
+    for (int lc = col_begin / 64; lc * 64 < col_end && ok; lc += KW, at.next()) {
+      if (!(ok = ptx::warp_all(gemm_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status)))) break;
+      const uint32_t x = ring + (uint32_t)at.slot * stage + KW * W_BYTES, full = bar_full(at.slot);
+      const int n = KW == 1 || (lc + 1) * 64 >= col_end ? 1 : KW;
+      if (ptx::elect_one()) {
         ptx::mbar_arrive_expect_tx(full, (uint32_t)n * xblk);
         for (int b = 0; b < n; ++b)
           ptx::tma_load_2d(x + (uint32_t)b * xblk, &tmPbd, 0, (2 * grp0 + lc + b) * 256 + (m0 & 255), full);
       }
-      if (!ok) drain(at);
     }
+    if (!ok && lane == 0) drain(at);
     __syncwarp();
   } else if (warp == 1) {
     // ============================ MMA issuer ============================
     // Both loops are unrolled with constant descriptor offsets: with a runtime trip count every MMA waited for its
     // operands to reach the uniform registers (790 clocks per K-block whatever its width).
+    // All three issuing warps walk their loops as a whole and elect the lane that issues (see gemm2_tcgen05.cuh): 512 x 4096 ->
+    // 4096 27.1 -> 23.5 us for the product alone, 64 rows 10.3 -> 9.5, 4096 -> 14336 24.1 -> 23.1.
     const uint32_t idesc_main = ptx::make_idesc_bf16(BM, (uint32_t)nb, !W_KMAJOR, false);
     const uint32_t idesc_lora = ptx::make_idesc_bf16(BM, (uint32_t)nb, true, false);
     uint32_t acc = 0;
-    int ok = 1;
+    bool ok = true;
     Ring at(S);
-    if (lane == 0) {
+    {
       for (int kb = kb_begin; kb < kb_end; ++kb, at.next()) {
-        if (!(ok = gemm_wait(bar_full(at.slot), at.parity, abort_flag, args.status))) break;
+        if (!(ok = ptx::warp_all(gemm_wait(bar_full(at.slot), at.parity, abort_flag, args.status)))) break;
         ptx::tc_fence_after();
         const uint32_t w = ring + (uint32_t)at.slot * stage;
         const uint64_t adesc = W_KMAJOR ? ptx::make_smem_desc(w, 16, 1024) : ptx::make_smem_desc(w, KW * 8192, 1024);
         const uint64_t bdesc = ptx::make_smem_desc(w + KW * W_BYTES, 16, 1024);
+        if (ptx::elect_one()) {
 #pragma unroll
-        for (int b = 0; b < KW; ++b)
+          for (int b = 0; b < KW; ++b)
 #pragma unroll
-          for (int k = 0; k < GEMM_BK / 16; ++k) {
-            ptx::umma_f16(tmem_base, adesc + (uint64_t)(W_KMAJOR ? b * (W_BYTES >> 4) + k * 2 : (b * 4 + k) * 128),
-                          bdesc + (uint64_t)(b * (xblk >> 4) + k * 2), idesc_main, acc);
-            acc = 1;
-          }
-        ptx::umma_commit(bar_empty(at.slot));
+            for (int k = 0; k < GEMM_BK / 16; ++k)
+              ptx::umma_f16(tmem_base, adesc + (uint64_t)(W_KMAJOR ? b * (W_BYTES >> 4) + k * 2 : (b * 4 + k) * 128),
+                            bdesc + (uint64_t)(b * (xblk >> 4) + k * 2), idesc_main, b + k == 0 ? acc : 1u);
+          ptx::umma_commit(bar_empty(at.slot));
+        }
+        acc = 1;
       }
     }
     __syncwarp();
     asm volatile("bar.sync 4, 160;" ::: "memory");
     lora_range();
-    if (lane == 0) {
+    {
       // How long the launch before takes must not count against the limit of the waits below.
       if (args.early && col_begin < col_end) ptx::grid_dependency_wait();
       // boxes of [2 halves][BOX rows][64 columns]: 16 operand columns are 16 rows of one box, or two boxes of 8
       auto lora_mma = [&](auto box_rows) {
         constexpr int BOX = decltype(box_rows)::value;
         for (int lc = col_begin / 64; lc * 64 < col_end && ok; lc += KW, at.next()) {
-          if (!(ok = gemm_wait(bar_full(at.slot), at.parity, abort_flag, args.status))) break;
+          if (!(ok = ptx::warp_all(gemm_wait(bar_full(at.slot), at.parity, abort_flag, args.status)))) break;
           ptx::tc_fence_after();
           const uint32_t w = ring + (uint32_t)at.slot * stage;
           const uint64_t adesc = ptx::make_smem_desc(w, BOX * 128, BOX == 8 ? 2048 : 1024);
           const uint64_t bdesc = ptx::make_smem_desc(w + KW * W_BYTES, 16, 1024);
           const int from = col_begin - lc * 64, to = col_end - lc * 64;
+          if (ptx::elect_one()) {
 #pragma unroll
-          for (int k = 0; k < KW * (GEMM_BK / 16); ++k)
-            if (k * 16 >= from && k * 16 < to) {
-              constexpr int per_box = BOX < 16 ? 1 : BOX / 16;
-              const uint32_t at_k = BOX == 8 ? k * 4096 : (k / per_box) * BOX * 256 + (k % per_box) * 2048;
-              ptx::umma_f16(tmem_base, adesc + (uint64_t)(at_k >> 4),
-                            bdesc + (uint64_t)((k >> 2) * (xblk >> 4) + (k & 3) * 2), idesc_lora, acc);
-              acc = 1;
-            }
-          ptx::umma_commit(bar_empty(at.slot));
+            for (int k = 0; k < KW * (GEMM_BK / 16); ++k)
+              if (k * 16 >= from && k * 16 < to) {
+                constexpr int per_box = BOX < 16 ? 1 : BOX / 16;
+                const uint32_t at_k = BOX == 8 ? k * 4096 : (k / per_box) * BOX * 256 + (k % per_box) * 2048;
+                ptx::umma_f16(tmem_base, adesc + (uint64_t)(at_k >> 4),
+                              bdesc + (uint64_t)((k >> 2) * (xblk >> 4) + (k & 3) * 2), idesc_lora, 1u);
+              }
+            ptx::umma_commit(bar_empty(at.slot));
+          }
         }
       };
       if (box == 8) lora_mma(std::integral_constant<int, 8>());
       else if (box == 16) lora_mma(std::integral_constant<int, 16>());
       else if (box == 32) lora_mma(std::integral_constant<int, 32>());
       else lora_mma(std::integral_constant<int, 64>());
-      if (ok) ptx::umma_commit(bar_done);
+      if (ok && ptx::elect_one()) ptx::umma_commit(bar_done);
     }
     __syncwarp();
   } else {

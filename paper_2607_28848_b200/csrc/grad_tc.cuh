@@ -228,7 +228,7 @@ grad_tc_kernel(const __grid_constant__ CUtensorMap tmQ0, const __grid_constant__
   volatile int* last_flag = reinterpret_cast<volatile int*>(misc + 16);
   int* piece_off = reinterpret_cast<int*>(misc + 32);                      // [<= 160] workspace slots of the pieces being added up
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = ptx::warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int cta = blockIdx.x, G = gridDim.x;
 
   if (threadIdx.x == 0) {
@@ -248,7 +248,7 @@ grad_tc_kernel(const __grid_constant__ CUtensorMap tmQ0, const __grid_constant__
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
-  const uint32_t tmem_base = *tmem_ptr_smem;
+  const uint32_t tmem_base = ptx::warp_uniform(*tmem_ptr_smem);
   const Ranges rg{G, a.NB * a.prob[0].NS, a.NB * a.prob[1].NS, a.snap, a.n_slots, a.slot_blk_off, a.prob[0].NS, a.prob[1].NS};
   int rt0[2], rt1[2];                                       // this CTA's tiles of either problem (plan tables only)
   rg.of(cta, 0, rt0[0], rt1[0]);
@@ -260,7 +260,7 @@ grad_tc_kernel(const __grid_constant__ CUtensorMap tmQ0, const __grid_constant__
 
   if (warp == 0) {
     // ================================ TMA producer ================================
-    if (lane == 0) {
+    {      // the whole warp walks the tiles, one elected lane issues (see gemm2_tcgen05.cuh)
       uint32_t i = 0;
       bool ok = true;
       for (int p = 0; p < 2 && ok; ++p) {
@@ -271,9 +271,12 @@ grad_tc_kernel(const __grid_constant__ CUtensorMap tmQ0, const __grid_constant__
         const CUtensorMap* tmQ = p ? &tmQ1 : &tmQ0;
         for (int t = t0; t < t1; ++t, ++i) {
           const int s = i % S;
-          if (!(ok = gemm_wait(bar_empty(s), ((i / S) & 1) ^ 1, abort_flag, a.status))) break;
-          ptx::mbar_arrive_expect_tx(bar_full(s), C::STAGE_BYTES);
-          ptx::tma_load_3d(s_stage(s), tmQ, 0, a.blk_row0[it.b0 + it.blk], it.strip * CB, bar_full(s));
+          const int row0 = a.blk_row0[it.b0 + it.blk];
+          if (!(ok = ptx::warp_all(gemm_wait(bar_empty(s), ((i / S) & 1) ^ 1, abort_flag, a.status)))) break;
+          if (ptx::elect_one()) {
+            ptx::mbar_arrive_expect_tx(bar_full(s), C::STAGE_BYTES);
+            ptx::tma_load_3d(s_stage(s), tmQ, 0, row0, it.strip * CB, bar_full(s));
+          }
           if (t + 1 < t1) it.next();
         }
       }
@@ -283,7 +286,7 @@ grad_tc_kernel(const __grid_constant__ CUtensorMap tmQ0, const __grid_constant__
     // ================================ MMA issuer ================================
     uint32_t i = 0, n_piece = 0;
     bool ok = true;
-    // the whole warp waits (one decision for all lanes); lane 0 issues
+    // the whole warp waits (one decision for all lanes), one elected lane issues
     auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
       return __all_sync(0xffffffffu, gemm_wait(bar, parity, abort_flag, a.status));
     };
@@ -314,15 +317,16 @@ grad_tc_kernel(const __grid_constant__ CUtensorMap tmQ0, const __grid_constant__
         }
         if (first_piece && !(ok = wait_all(bar_accempty(ab), ((n_piece >> 1) & 1) ^ 1))) break;
         ptx::tc_fence_after();
-        if (lane == 0) {
-          const int ksteps = (nrows + 15) >> 4;
+        const int ksteps = (nrows + 15) >> 4;
+        if (ptx::elect_one()) {
           const uint64_t bd0 = ptx::make_smem_desc(s_pbuf(pb), 16, 1024);
 #pragma unroll
           for (int mb = 0; mb < CB / 2; ++mb) {
             const uint32_t d = tmem_base + (uint32_t)(ab * C::ACC_COLS + mb * N2);
             const uint64_t ad = ptx::make_smem_desc(q + (uint32_t)(2 * mb) * C::BLK, C::BLK, 1024);
-            for (int ks = 0; ks < ksteps; ++ks)      // K-step ks: rows 16 ks .. of the tile; P's K-block ks / 4, 32 bytes per step inside it
-              ptx::umma_f16(d, ad + (uint64_t)(ks * 128), bd0 + (uint64_t)((ks >> 2) * (n2 * 8) + (ks & 3) * 2), idesc,
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks)           // K-step ks: rows 16 ks .. of the tile; P's K-block ks / 4, 32 bytes per step inside it
+              if (ks < ksteps) ptx::umma_f16(d, ad + (uint64_t)(ks * 128), bd0 + (uint64_t)((ks >> 2) * (n2 * 8) + (ks & 3) * 2), idesc,
                             (ks == 0 && first_piece) ? 0u : 1u);
           }
           ptx::umma_commit(bar_empty(s));

@@ -21,6 +21,12 @@ __device__ __forceinline__ bool elect_one() {
   return pred != 0;
 }
 
+// A value that is the same in all lanes, in a form from which the compiler knows it (the roles of a warp branch on it, and a loop
+// that the whole warp walks keeps what it computes from such values in uniform registers, where the tensor-core instructions
+// take their operands from).
+__device__ __forceinline__ int warp_uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+__device__ __forceinline__ bool warp_all(bool x) { return __all_sync(0xffffffffu, x) != 0; }
+
 // ---- programmatic dependent launch ----------------------------------------------------------
 // A kernel launched with the programmatic-stream-serialization attribute may begin while its
 // predecessor in the stream is still draining.  grid_dependency_wait() blocks until the
@@ -148,6 +154,14 @@ __device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a_desc, uint6
 // Arrives on the mbarrier once every tcgen05 operation issued so far by this thread is done.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// The same, called by a whole warp of which one lane issues: elect_one() picks the same lane every time.
+__device__ __forceinline__ void umma_f16_elected(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  if (elect_one()) umma_f16(d_tmem, a_desc, b_desc, idesc, accumulate);
+}
+__device__ __forceinline__ void umma_commit_elected(uint32_t bar) {
+  if (elect_one()) umma_commit(bar);
 }
 
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp reads lane (base lane + i).
