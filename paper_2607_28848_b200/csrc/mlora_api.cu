@@ -1191,7 +1191,7 @@ mlora_status_t simt_shrink(mlora_ctx* ctx, const T* In, int64_t ld_in, int D, in
   const int64_t warps = (int64_t)n_rows * R;
   const int blocks = (int)((warps * 32 + 255) / 256);
   LaunchScope scope(ctx, st, KIND_SIMT);
-  simt::shrink_kernel<T><<<blocks, 256, 0, st>>>(In, ld_in, D, R, P_all, scale, ds.row_adapter, ds.row_save, Out,
+  launch_pdl(scope.slot < 0, simt::shrink_kernel<T>, dim3(blocks), dim3(256), 0, st, In, ld_in, D, R, P_all, scale, ds.row_adapter, ds.row_save, Out,
                                                  x_save, u_save, save_base, n_rows, n_adapters, drop);
   return scope.done();
 }
@@ -1204,21 +1204,95 @@ mlora_status_t simt_gemm(mlora_ctx* ctx, const T* In, int64_t ld_in, const T* W,
   if (cancelled(ctx)) return MLORA_CANCELLED;
   const dim3 grid = simt::gemm_grid(M, N), block(32, simt::GEMM_ROWS);
   LaunchScope scope(ctx, st, KIND_SIMT);
-  simt::gemm_lora_kernel<T, W_KMAJOR><<<grid, block, 0, st>>>(In, ld_in, W, ldw, L_all, P, scale, ds.row_adapter, Out,
+  launch_pdl(scope.slot < 0, simt::gemm_lora_kernel<T, W_KMAJOR>, grid, block, 0, st, In, ld_in, W, ldw, L_all, P, scale, ds.row_adapter, Out,
                                                               ld_out, M, N, K, R, n_adapters, drop);
   return scope.done();
 }
 
 template <typename T>
-mlora_status_t simt_grad(mlora_ctx* ctx, const mlora_plan* p, const float* P, int R, const float* scale, const T* Q,
-                         int64_t ldq, int D, float* G, int accumulate, const DropArgs& drop, cudaStream_t st) {
-  const int n_slots = (int)p->h.ft_adapters.size();
-  if (n_slots <= 0) return MLORA_OK;
+simt::GradTask<T> simt_grad_task(const mlora_plan* p, const float* P, int R, const float* scale, const T* Q, int64_t ldq, int D, float* G,
+                                 int accumulate, const DropArgs& drop) {
+  return simt::GradTask<T>{P, scale, Q, ldq, G, R, D, (int32_t)p->h.ft_adapters.size(), accumulate,
+                           p->slot_chunk_off, p->chunk_row0, p->chunk_nrows, p->slot_adapter, drop};
+}
+template <typename T>
+mlora_status_t simt_grad(mlora_ctx* ctx, const simt::GradTask<T>& g, cudaStream_t st) {
+  if (g.n_slots <= 0) return MLORA_OK;
   if (cancelled(ctx)) return MLORA_CANCELLED;
-  dim3 grid((D + 127) / 128, R, n_slots);
   LaunchScope scope(ctx, st, KIND_SIMT);
-  simt::grad_kernel<T><<<grid, 128, 0, st>>>(P, R, scale, Q, ldq, D, G, p->slot_chunk_off, p->chunk_row0,
-                                             p->chunk_nrows, p->slot_adapter, accumulate, drop);
+  launch_pdl(scope.slot < 0, simt::grad_kernel<T>, dim3((g.D + 127) / 128, g.R, g.n_slots), dim3(128), 0, st, g);
+  return scope.done();
+}
+
+// Small fp32 layers run in fewer launches (simt.cuh): where the rank-R products that every column block repeats cost less than
+// the launches.  Forward + backward of d -> d layers, six launches / three, us (16 rows, then 160): d 64 rank 8 21.2 / 15.2, 21.9 / 15.3,
+// rank 32 21.2 / 15.5, 23.1 / 18.0; d 256 rank 8 21.7 / 18.2, 29.8 / 21.5, but rank 16 21.0 / 22.2; d 512 rank 4 25.7 / 26.0, rank 8
+// 25.4 / 28.9.  Rows are as far as was measured: 256 rows all to be tuned at d 256, rank 8 50.0 / 43.9.
+bool small_layer(const mlora_ctx* ctx, const mlora_layer_t* L, int rows) {
+  const int d = L->d_in > L->d_out ? L->d_in : L->d_out;
+  return L->dtype == MLORA_F32 && ctx->gemm_path == 0 && d <= 256 && L->rank * d <= 2048 && rows <= 256;
+}
+// Rows of `cols` floats, `ld` apart.  The launches that were merged used to run one behind the other, so a caller whose output
+// lies over an operand of the launch before it keeps the separate ones.
+struct Span {
+  uintptr_t lo, hi;
+  Span(const void* p, int64_t rows, int64_t ld, int64_t cols) : lo((uintptr_t)p), hi((uintptr_t)p) {
+    if (p && rows > 0) hi += (uintptr_t)(((rows - 1) * ld + cols) * 4);
+  }
+};
+inline bool apart(const Span& a, const Span& b) { return a.hi <= b.lo || b.hi <= a.lo; }
+bool forward_small_fits(const mlora_ctx* ctx, const mlora_layer_t* L, const mlora_plan* p, const void* Y, int64_t ldy, const void* x_save,
+                        const float* u_save, int64_t base) {
+  if (!small_layer(ctx, L, p->h.n_rows)) return false;
+  const int64_t ar = (int64_t)L->n_adapters * L->rank, ft = p->h.ft_rows;
+  const Span y(Y, p->h.n_rows, ldy, L->d_out), rows(x_save ? (const float*)x_save + base * L->d_in : nullptr, ft, L->d_in, L->d_in);
+  const Span u(u_save ? u_save + base * L->rank : nullptr, ft, L->rank, L->rank);
+  const Span A(L->A_all, ar, L->d_in, L->d_in), B(L->B_all, ar, L->d_out, L->d_out), W(L->W, L->d_in, L->ldw, L->d_out);
+  return apart(y, A) && apart(y, rows) && apart(y, u) && apart(rows, A) && apart(rows, B) && apart(rows, W) && apart(u, A) && apart(u, B) &&
+         apart(u, W);
+}
+bool backward_small_fits(const mlora_ctx* ctx, const mlora_layer_t* L, const mlora_plan* p, const void* dY, int64_t lddy, const void* x_save,
+                         const float* dA, const float* dB, const void* dX, int64_t lddx) {
+  const int T = p->h.ft_rows;
+  if (!small_layer(ctx, L, T)) return false;
+  const int64_t ar = (int64_t)L->n_adapters * L->rank, sr = (int64_t)p->h.ft_adapters.size() * L->rank;
+  const Span gA(dA, sr, L->d_in, L->d_in), gB(dB, sr, L->d_out, L->d_out), x(dX, T, lddx, L->d_in);
+  const Span A(L->A_all, ar, L->d_in, L->d_in), B(L->B_all, ar, L->d_out, L->d_out), W(L->W, L->d_in, L->ldw, L->d_out);
+  const Span y(dY, T, lddy, L->d_out), rows(x_save, T, L->d_in, L->d_in);
+  return apart(gB, B) && apart(gB, y) && apart(gA, y) && apart(gA, W) && apart(gA, A) && apart(gA, rows) && apart(x, rows) && apart(x, gA);
+}
+mlora_status_t forward_small(mlora_ctx* ctx, const mlora_layer_t* L, const mlora_plan* p, const float* X, int64_t ldx, float* Y, int64_t ldy,
+                             float* x_save, float* u_save, int64_t save_base, cudaStream_t st) {
+  if (cancelled(ctx)) return MLORA_CANCELLED;
+  LaunchScope scope(ctx, st, KIND_SIMT);
+  launch_pdl(scope.slot < 0, simt::small_forward_kernel<float>, simt::gemm_grid(p->h.n_rows, L->d_out), dim3(32, simt::GEMM_ROWS), 0, st, X, ldx, (const float*)L->W, L->ldw, (const float*)L->A_all, (const float*)L->B_all, L->scale, p->fwd.row_adapter, p->fwd.row_save, Y, ldy,
+      x_save, u_save, save_base, p->h.n_rows, L->d_out, L->d_in, L->rank, ctx->drop);
+  return scope.done();
+}
+mlora_status_t backward_small(mlora_ctx* ctx, const mlora_layer_t* L, const mlora_plan* p, const float* dY, int64_t lddy, const float* x_save,
+                              const float* u_save, float* dA, float* dB, float* dX, int64_t lddx, int accumulate, cudaStream_t st) {
+  const int T = p->h.ft_rows, R = L->rank;
+  const DropArgs off = {0, 0, 1.0f};
+  const auto gB = simt_grad_task<float>(p, u_save, R, L->scale, dY, lddy, L->d_out, dB, accumulate, off);
+  const auto gA = simt_grad_task<float>(p, ctx->ws_p, R, nullptr, x_save, L->d_in, L->d_in, dA, accumulate, ctx->drop);
+  auto grad_blocks = [](const simt::GradTask<float>& g) { return (g.D + 255) / 256 * g.R * g.n_slots; };
+  const dim3 block(32, simt::GEMM_ROWS);
+  if (cancelled(ctx)) return MLORA_CANCELLED;
+  {
+    LaunchScope scope(ctx, st, KIND_SIMT);
+    const int v_blocks = (T * R + simt::GEMM_ROWS - 1) / simt::GEMM_ROWS;
+    launch_pdl(scope.slot < 0, simt::small_backward_v_kernel<float>, dim3(v_blocks + grad_blocks(gB)), block, 0, st, dY, lddy, L->d_out, (const float*)L->B_all, L->scale,
+                                                                                       p->bwd.row_adapter, ctx->ws_p, T, grad_blocks(gB), gB);
+    const mlora_status_t s = scope.done();
+    if (s != MLORA_OK) return s;
+  }
+  if (cancelled(ctx)) return MLORA_CANCELLED;
+  LaunchScope scope(ctx, st, KIND_SIMT);
+  const dim3 g = simt::gemm_grid(T, L->d_in);
+  const int tiles = dX ? (int)(g.x * g.y) : 0;
+  launch_pdl(scope.slot < 0, simt::small_backward_x_kernel<float>, dim3(tiles + grad_blocks(gA)), block, 0, st, dY, lddy, (const float*)L->W, L->ldw, (const float*)L->A_all,
+                                                                                  ctx->ws_p, p->bwd.row_adapter, dX, lddx, T, L->d_in, L->d_out,
+                                                                                  grad_blocks(gA), gA);
   return scope.done();
 }
 
@@ -1242,10 +1316,10 @@ mlora_status_t backward_simt(mlora_ctx* ctx, const mlora_layer_t* L, const mlora
   mlora_status_t s = simt_shrink<T>(ctx, (const T*)dY, lddy, L->d_out, L->rank, (const T*)L->B_all, L->scale, p->bwd,
                                     ctx->ws_p, (T*)nullptr, nullptr, 0, Tft, L->n_adapters, off, st);
   if (s != MLORA_OK) return s;
-  if ((s = simt_grad<T>(ctx, p, u_save, L->rank, L->scale, (const T*)dY, lddy, L->d_out, dB, accumulate, off, st)) != MLORA_OK)
+  if ((s = simt_grad(ctx, simt_grad_task<T>(p, u_save, L->rank, L->scale, (const T*)dY, lddy, L->d_out, dB, accumulate, off), st)) != MLORA_OK)
     return s;
-  if ((s = simt_grad<T>(ctx, p, ctx->ws_p, L->rank, nullptr, (const T*)x_save, L->d_in, L->d_in, dA, accumulate, ctx->drop,
-                        st)) != MLORA_OK)
+  if ((s = simt_grad(ctx, simt_grad_task<T>(p, ctx->ws_p, L->rank, nullptr, (const T*)x_save, L->d_in, L->d_in, dA, accumulate, ctx->drop),
+                     st)) != MLORA_OK)
     return s;
   if (dX)
     s = simt_gemm<T, true>(ctx, (const T*)dY, lddy, (const T*)L->W, L->ldw, (const T*)L->A_all, ctx->ws_p, nullptr,
@@ -1765,6 +1839,8 @@ mlora_status_t mlora_mixed_forward(mlora_ctx* ctx, const mlora_layer_t* L, const
   // calling thread (a framework's worker threads do not always have one)
   if (cudaSetDevice(ctx->device) != cudaSuccess) return MLORA_ERR_CUDA;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
+  if (L->dtype == MLORA_F32 && forward_small_fits(ctx, L, p, Y, ldy, x_save, u_save, save_row_base))
+    return forward_small(ctx, L, p, (const float*)X, ldx, (float*)Y, ldy, (float*)x_save, u_save, save_row_base, st);
   if (L->dtype == MLORA_F32)
     return forward_simt<float>(ctx, L, p, X, ldx, Y, ldy, x_save, u_save, save_row_base, st);
   if (ldx % 8 || ldy % 8 || !aligned16(X) || !aligned16(Y) || (x_save && !aligned16(x_save))) return MLORA_ERR_UNSUPPORTED;
@@ -1809,6 +1885,8 @@ mlora_status_t mlora_backward(mlora_ctx* ctx, const mlora_layer_t* L, const mlor
   // calling thread (a framework's worker threads do not always have one)
   if (cudaSetDevice(ctx->device) != cudaSuccess) return MLORA_ERR_CUDA;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
+  if (L->dtype == MLORA_F32 && backward_small_fits(ctx, L, p, dY, lddy, x_save, dA, dB, dX, lddx))
+    return backward_small(ctx, L, p, (const float*)dY, lddy, (const float*)x_save, u_save, dA, dB, (float*)dX, lddx, accumulate, st);
   if (L->dtype == MLORA_F32)
     return backward_simt<float>(ctx, L, p, dY, lddy, x_save, u_save, dA, dB, dX, lddx, accumulate, st);
   if (lddy % 8 || (dX && lddx % 8) || !aligned16(dY) || !aligned16(x_save) || (dX && !aligned16(dX)) ||
@@ -1934,8 +2012,8 @@ mlora_status_t mlora_adamw_update(mlora_ctx* ctx, const mlora_layer_t* L, const 
   int blocks = (int)((widest + 255) / 256);
   blocks = blocks < 4 * ctx->sm_count ? blocks : 4 * ctx->sm_count;
   LaunchScope scope(ctx, st, KIND_ADAMW);
-  if (L->dtype == MLORA_F32) simt::adamw_kernel<float><<<dim3(blocks, 2), 256, 0, st>>>(a);
-  else simt::adamw_kernel<__nv_bfloat16><<<dim3(blocks, 2), 256, 0, st>>>(a);
+  if (L->dtype == MLORA_F32) launch_pdl(scope.slot < 0, simt::adamw_kernel<float>, dim3(blocks, 2), dim3(256), 0, st, a);
+  else launch_pdl(scope.slot < 0, simt::adamw_kernel<__nv_bfloat16>, dim3(blocks, 2), dim3(256), 0, st, a);
   return scope.done();
 }
 
