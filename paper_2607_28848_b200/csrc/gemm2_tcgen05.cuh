@@ -29,6 +29,8 @@
 
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "gemm_tcgen05.cuh"
 #include "ptx.cuh"
 
@@ -142,7 +144,6 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
                   const __grid_constant__ CUtensorMap tmL, const __grid_constant__ CUtensorMap tmOut,
                   const __grid_constant__ CUtensorMap tmPbd, const GemmArgs args) {
   static_assert(R == 8 || R == 16 || R == 32 || R == 64 || R == 128, "rank");
-  constexpr int GPC = R <= 64 ? 64 / R : 1;          // groups per 64-wide low-rank block
   constexpr int S = GEMM2_STAGES;
 
   extern __shared__ uint8_t smem_raw[];
@@ -212,10 +213,6 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
 
   if (warp == 0) {
     // ============================ TMA producer (both CTAs) ============================
-    // One elected lane issues the main loads; the low-rank stages are issued by all lanes, one
-    // adapter group per lane, from a copy of the tile's adapter list in shared memory, so that
-    // the list costs one memory latency per tile rather than one per group.
-    int32_t* ga_smem = reinterpret_cast<int32_t*>(smem_gen + (sMisc - smem_base) + 64);   // 256 entries
     uint32_t it = 0;
     bool ok = true;
     for (int ui = u_begin; ui < u_end && ok; ui += u_step) {
@@ -234,12 +231,24 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
       const int lc_begin = (int)((long long)ks * LC / SK), lc_end = (int)((long long)(ks + 1) * LC / SK);
       const int kb_begin = (int)((long long)ks * KB / SK), kb_end = (int)((long long)(ks + 1) * KB / SK);
       const int chunk_base = args.lora_enabled ? args.tile_grp_off[mt] : 0;   // chunk slot = 2 * this + lc
-      int32_t ga_reg[8];                                  // G <= 256 adapters of the pair tile
-      {
-        const int32_t* ga = args.grp_adapter + (args.lora_enabled ? args.tile_grp_off[mt] : 0);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) ga_reg[j] = (lane + 32 * j < G) ? ga[lane + 32 * j] : 0;
-      }
+      // Rows of the adapters' matrices, one box per lane, the next 32 already on their way (one memory latency per 32 boxes).
+      // A box brings both 64-column halves of this CTA's columns, [half][box rows][64], and the boxes are issued one after the other by
+      // an elected lane: each half from a lane of its own cost ~150 clocks, five to nine of them a K-block and more than its MMAs
+      // (512 decode rows of 128 adapters of rank 32, 5120 -> 13824: 134.8 us the call, 127.0 now).
+      const int n_boxes = ranked ? pc_end - pc_base : (R > 64 ? 2 * G : G), per_grp = R > 64 ? R / 64 : 1;
+      auto box_rows = [&](int j0) -> int {
+        const int j = j0 + lane;
+        if (j >= n_boxes) return 0;
+        if (ranked) {
+          const int src = args.piece_src[pc_base + j];
+          return (src >> 8) * R + (src & 255) * 16;
+        }
+        return args.grp_adapter[chunk_base + j / per_grp] * R + (j % per_grp) * 64;
+      };
+      const int box = ranked ? 16 : (R < 64 ? R : 64), per = 64 / box;
+      int batch = (lc_begin * per) & ~31;
+      int cur = 0, next = 0;
+      if (lc_end > lc_begin) { cur = box_rows(batch); next = box_rows(batch + 32); }
       for (int kb = kb_begin; kb < kb_end; ++kb, ++it) {
         const int s = it % S;
         ok = ptx::warp_all(gemm2_wait(bar_empty(s), ((it / S) & 1) ^ 1, abort_flag, args.status));
@@ -258,58 +267,23 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
       // blocks or not: from here on a slot may come free, or an accumulator be read, only after it, and how long it takes
       // must not count against the limit of a wait inside this kernel.
       if (args.early && ui == u_begin) ptx::grid_dependency_wait();
-      if (lc_end > lc_begin && !ranked) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (lane + 32 * j < G) ga_smem[lane + 32 * j] = ga_reg[j];
-        __syncwarp();
-      }
-      // ranked plans: the pieces of eight chunks at a time, one per lane (one memory latency per eight chunks, the next
-      // eight already on their way)
-      auto piece_batch = [&](int first_chunk) -> int {
-        const int idx = pc_base + 4 * first_chunk + lane;
-        return (ranked && idx < pc_end) ? args.piece_src[idx] : 0;
-      };
-      int pb_chunk0 = lc_begin & ~7;
-      int pb_cur = piece_batch(pb_chunk0), pb_next = piece_batch(pb_chunk0 + 8);
       for (int lc = lc_begin; lc < lc_end; ++lc, ++it) {
         const int s = it % S;
-        if (lane == 0) ok = gemm2_wait(bar_empty(s), ((it / S) & 1) ^ 1, abort_flag, args.status);
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        ok = ptx::warp_all(gemm2_wait(bar_empty(s), ((it / S) & 1) ^ 1, abort_flag, args.status));
         if (!ok) break;
-        if (ranked && (lc & ~7) != pb_chunk0) { pb_chunk0 += 8; pb_cur = pb_next; pb_next = piece_batch(pb_chunk0 + 8); }
-        const int piece_of_lane = __shfl_sync(0xffffffffu, pb_cur, 4 * (lc & 7) + (lane & 3));
+        if (((lc * per) & ~31) != batch) { batch += 32; cur = next; next = box_rows(batch + 32); }
+        const int j0 = lc * per, j1 = n_boxes < j0 + per ? n_boxes : j0 + per;
+        const int n = (R == 8 && !ranked && ((j1 - j0) & 1)) ? j1 - j0 + 1 : j1 - j0;      // rank 8: a half-filled MMA step repeats the last group
         const uint32_t a = sA0 + s * GEMM2_STAGE_BYTES, b = a + GEMM2_A_BYTES;
         const uint32_t full = ptx::map_to_cta(bar_full(s), 0);
-        // A operand: this CTA's 128 rows of chunk lc of the tile's block-diagonal low-rank matrix
-        if (lane == 0) ptx::tma2_load_2d(a, &tmPbd, 0, (2 * chunk_base + lc) * 256 + (int)rank * 128, full);
-        if (ranked) {
-          // B operand: up to four 16-row pieces of the adapters' matrices, one per lane (tmL has 16-row boxes here)
-          const int left = pc_end - (pc_base + 4 * lc);
-          const int np = left < 4 ? left : 4;
-          if (leader && lane == 0) ptx::mbar_arrive_expect_tx(bar_full(s), 2u * (GEMM2_A_BYTES + (uint32_t)np * 16u * 128u * 2u));
-          if (lane < np) {
-            const int src = piece_of_lane;
-            const int brow = (src >> 8) * R + (src & 255) * 16;
-#pragma unroll
-            for (int nb = 0; nb < 2; ++nb)
-              ptx::tma2_load_3d(b + nb * 8192 + lane * 16 * 128, &tmL, 0, brow, (nh >> 6) + nb, full);
-          }
-        } else if (R <= 64) {
-          const int g0 = lc * GPC;
-          const int ng = G - g0 < GPC ? G - g0 : GPC;
-          const int ngl = (R == 8 && (ng & 1)) ? ng + 1 : ng;   // rank 8: pad a half-filled MMA step
-          if (leader && lane == 0) ptx::mbar_arrive_expect_tx(bar_full(s), 2u * (GEMM2_A_BYTES + (uint32_t)ngl * R * 128u * 2u));
-          if (lane < ngl) {
-            const int adapter = ga_smem[g0 + (lane < ng ? lane : ng - 1)];
-#pragma unroll
-            for (int nb = 0; nb < 2; ++nb)
-              ptx::tma2_load_3d(b + nb * 8192 + lane * R * 128, &tmL, 0, adapter * R, (nh >> 6) + nb, full);
-          }
-        } else {
-          if (leader && lane == 0) ptx::mbar_arrive_expect_tx(bar_full(s), 2u * (GEMM2_A_BYTES + 64u * 128u * 2u));
-          if (lane < 2)
-            ptx::tma2_load_3d(b + lane * 8192, &tmL, 0, ga_smem[lc >> 1] * R + (lc & 1) * 64, (nh >> 6) + lane, full);
+        if (ptx::elect_one()) {
+          if (leader) ptx::mbar_arrive_expect_tx(bar_full(s), 2u * (GEMM2_A_BYTES + (uint32_t)(n * box) * 256u));
+          // A operand: this CTA's 128 rows of chunk lc of the tile's block-diagonal low-rank matrix
+          ptx::tma2_load_2d(a, &tmPbd, 0, (2 * chunk_base + lc) * 256 + (int)rank * 128, full);
+        }
+        for (int i = 0; i < n; ++i) {
+          const int brow = __shfl_sync(0xffffffffu, cur, (j0 + i < j1 ? j0 + i : j1 - 1) & 31);
+          if (ptx::elect_one()) ptx::tma2_load_3d(b + (uint32_t)(i * box) * 256u, &tmL, 0, brow, nh >> 6, full);
         }
       }
     }
@@ -360,23 +334,31 @@ gemm2_lora_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constan
         if (args.early && ui == u_begin) ptx::grid_dependency_wait();      // as the producer
         const int LC = (lcols + 63) / 64;
         const int lc_begin = (int)((long long)ks * LC / SK), lc_end = (int)((long long)(ks + 1) * LC / SK);
-        for (int lc = lc_begin; lc < lc_end; ++lc, ++it) {
-          const int s = it % S;
-          if (!(ok = ptx::warp_all(gemm2_wait(bar_full(s), (it / S) & 1, abort_flag, args.status)))) break;
-          ptx::tc_fence_after();
-          const uint32_t a = sA0 + s * GEMM2_STAGE_BYTES, b = a + GEMM2_A_BYTES;
-          const uint64_t adesc = ptx::make_smem_desc(a, 16, 1024);
-          const uint64_t bdesc = ptx::make_smem_desc(b, 8192, 1024);
-          int ksteps = (lcols - lc * 64 + 15) / 16;
-          ksteps = ksteps < 4 ? ksteps : 4;
-          if (ptx::elect_one()) {
+        // boxes of [2 halves][BOX rows][64 columns]: 16 operand columns are 16 rows of one box, or two boxes of 8
+        auto lora_mma = [&](auto box_rows) {
+          constexpr int BOX = decltype(box_rows)::value;
+          for (int lc = lc_begin; lc < lc_end; ++lc, ++it) {
+            const int s = it % S;
+            if (!(ok = ptx::warp_all(gemm2_wait(bar_full(s), (it / S) & 1, abort_flag, args.status)))) break;
+            ptx::tc_fence_after();
+            const uint32_t a = sA0 + s * GEMM2_STAGE_BYTES, b = a + GEMM2_A_BYTES;
+            const uint64_t adesc = ptx::make_smem_desc(a, 16, 1024);
+            const uint64_t bdesc = ptx::make_smem_desc(b, BOX * 128, BOX == 8 ? 2048 : 1024);
+            const int ksteps = (lcols - lc * 64 + 15) / 16;
+            if (ptx::elect_one()) {
 #pragma unroll
-            for (int ks = 0; ks < GEMM_BK / 16; ++ks)
-              if (ks < ksteps) ptx::umma2_f16(d_tmem, adesc + (uint64_t)(ks * 2), bdesc + (uint64_t)(ks * 128), idesc_lora, ks == 0 ? acc : 1u);
-            ptx::umma2_commit_both(bar_empty(s));
+              for (int k = 0; k < GEMM_BK / 16; ++k)
+                if (k < ksteps) {
+                  constexpr int per_box = BOX < 16 ? 1 : BOX / 16;
+                  const uint32_t at_k = BOX == 8 ? k * 4096 : (k / per_box) * BOX * 256 + (k % per_box) * 2048;
+                  ptx::umma2_f16(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(at_k >> 4), idesc_lora, 1u);
+                }
+              ptx::umma2_commit_both(bar_empty(s));
+            }
           }
-          acc = 1;
-        }
+        };
+        if (R > 8 && args.piece_src != nullptr) lora_mma(std::integral_constant<int, 16>());
+        else lora_mma(std::integral_constant<int, (R < 64 ? R : 64)>());
         if (!ok) break;
         if (ptx::elect_one()) ptx::umma2_commit_both(bar_tfull(buf));
       }

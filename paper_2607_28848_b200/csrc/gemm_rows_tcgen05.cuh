@@ -169,11 +169,11 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant
       const int j0 = box_begin > lc * per ? box_begin : lc * per, j1 = box_end < (lc + KW) * per ? box_end : (lc + KW) * per;
       const int n = box == 8 ? (j1 - j0 + 1) & ~1 : j1 - j0;     // rank 8: a half-filled MMA step repeats the last group (its operand columns are zero)
       const uint32_t w = ring + (uint32_t)at.slot * stage, full = bar_full(at.slot);
-      if (lane == 0) ptx::mbar_arrive_expect_tx(full, (uint32_t)(n * box) * 256u);
-      __syncwarp();
-      if (lane < n) {                      // one box per lane, both 64-column halves: [half][box rows][64]
-        const int j = j0 + lane;
-        ptx::tma_load_3d(w + (uint32_t)((j - lc * per) * box) * 256u, &tmL, 0, box_row[j < j1 ? j : j1 - 1], n0 >> 6, full);
+      if (ptx::elect_one()) ptx::mbar_arrive_expect_tx(full, (uint32_t)(n * box) * 256u);
+      const int mine = lane < n ? box_row[j0 + lane < j1 ? j0 + lane : j1 - 1] : 0;
+      for (int i = 0; i < n; ++i) {        // one box after the other, both 64-column halves: [half][box rows][64]
+        const int brow = __shfl_sync(0xffffffffu, mine, i);
+        if (ptx::elect_one()) ptx::tma_load_3d(w + (uint32_t)((j0 + i - lc * per) * box) * 256u, &tmL, 0, brow, n0 >> 6, full);
       }
     }
     if (!ok && lane == 0) drain(at);

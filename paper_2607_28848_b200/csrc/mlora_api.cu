@@ -1120,7 +1120,8 @@ mlora_status_t gemm_bf16(mlora_ctx* ctx, const mlora_layer_t* L, const RowSpace&
   }
   const int R = L->rank;
   const bool ranked = ds.piece_src != nullptr && ctx->gemm_pairs;    // B-side rows of the low-rank blocks come as 16-row pieces
-  if ((s = make_tmap_bf16_blocked(ctx, &tL, L_all, (uint64_t)L->n_adapters * R, N, N, ranked ? 16 : (R < 64 ? R : 64), 1)) != MLORA_OK)
+  // (the two-SM kernel loads both 64-column halves of a CTA's columns in one box)
+  if ((s = make_tmap_bf16_blocked(ctx, &tL, L_all, (uint64_t)L->n_adapters * R, N, N, ranked ? 16 : (R < 64 ? R : 64), ctx->gemm_pairs ? 2 : 1)) != MLORA_OK)
     return s;
   if ((s = make_tmap_bf16(ctx, &tOut, Out, N, M, ld_out, 64, 32)) != MLORA_OK) return s;
   GemmArgs g;
