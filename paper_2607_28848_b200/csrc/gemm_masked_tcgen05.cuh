@@ -1,0 +1,463 @@
+// Input gradient under LoRA dropout (see gemm_tcgen05.cuh for the operator without it):
+//
+//      dX[m, n] = (dY W^T)[m, n] + keep(m, n) / (1 - p) (V A_{a(m)})[m, n]
+//
+// The mask acts on the low-rank term element by element, so that term has an accumulator of its own in tensor memory and the
+// epilogue adds what is kept.  Before, a launch behind the product read and wrote dX once more and computed V A on the CUDA cores:
+// 8 us of a backward of 256 rows 4096 -> 4096 at rank 16, 100 us at rank 64 with 15 adapters, and dX was rounded twice.  V enters as
+// bf16 head and remainder (16 bits of mantissa), both against the same rows of the adapters.
+//
+// 256 weight columns of a CTA pair are the MMA's M side, 128 per CTA, the batch rows its N side, as many as the batch needs; a pair
+// has one tile of up to 256 rows, and more rows than the pairs hold at once take several launches.  Where there are fewer tiles than
+// pairs, K is cut over the pairs of a cluster (up to four), which add their fp32 sums over distributed shared memory in slice order.
+//
+// Two-SM synchronisation as in gemm2_tcgen05.cuh (full[] in the leader counts both CTAs' bytes, empty[] is signalled in both by
+// tcgen05.commit), start before the end of the launch in front (`early`) as in gemm_rows_tcgen05.cuh.
+//
+// Warp roles (192 threads): warp 0 loads, warp 1 issues the MMAs (leader) and owns tensor memory, warps 2-5 look up the tile's
+// low-rank tables and write the result.  Every wait is bounded, and all threads meet in the block and cluster barriers on
+// every path.
+#pragma once
+
+#include <cuda.h>
+
+#include <type_traits>
+
+#include "dropout.cuh"
+#include "gemm2_tcgen05.cuh"
+#include "gemm_rows_tcgen05.cuh"
+#include "gemm_tcgen05.cuh"
+#include "ptx.cuh"
+#include "ring.h"
+
+namespace mlora {
+namespace masked {
+
+constexpr int BN = 256;                              // output columns of a pair's tile (UMMA M): 128 per CTA
+constexpr int THREADS = 192;
+constexpr uint32_t W_BYTES = 128 * GEMM_BK * 2;      // 16 KiB: this CTA's columns of one K-block of the weight
+constexpr int MAX_STAGES = 8;
+constexpr uint32_t RING_BYTES = 192u << 10;
+constexpr uint32_t STAGING_BYTES = 2 * 8192;         // two buffers of [2 column halves][32 rows][64] bf16
+constexpr uint32_t SMEM_BYTES = RING_BYTES + STAGING_BYTES + 1024;
+
+struct Args {
+  int32_t M, N, K;              // batch rows, output columns, contraction
+  int32_t nb;                   // rows of a tile (the MMA's N): a multiple of 16, at most 256
+  int32_t col_tiles;
+  int32_t rt0;                  // first row tile of this launch
+  int32_t stages;               // ring depth
+  int32_t slices;               // pairs of a cluster = K slices of a tile: 1 to 4
+  int32_t R;                    // rank
+  int32_t early;                // 1: weight and input rows may be read before the dependency wait
+  const int32_t* tile_grp_off;  // groups of each 256-row tile of the batch, and their adapters
+  const int32_t* grp_adapter;
+  const int32_t* tile_cols;     // plans made with per-adapter ranks (else null): columns of a tile's low-rank operand, first
+  const int32_t* grp_col;          // column of each group,
+  const int32_t* tile_piece_off;   // and its B side as 16-row pieces of the adapters' matrices
+  const int32_t* piece_src;
+  DropArgs drop;                // the dropout that the low-rank term passes through
+  int32_t rest;                 // chunk slots between a value's place in the low-rank operand and its remainder's
+  int32_t* status;
+};
+
+__host__ __device__ __forceinline__ uint32_t stage_bytes(int nb) { return W_BYTES + (uint32_t)nb * 64u; }
+// Rows of a tile that one of its slices finishes: whole boxes of 16.
+__host__ __device__ __forceinline__ int slice_rows(int nb, int slices) { return (nb / 16 + slices - 1) / slices * 16; }
+
+// The low-rank operand is laid out per 256-row tile of the batch, two of which the rows of a tile here may straddle: they meet it
+// in up to two segments, each with the K-blocks of its own 256-row tile and MMAs over its own rows only.
+struct Segment {
+  int32_t row0, rows;           // batch rows [row0, row0 + rows)
+  int32_t at;                   // accumulator column of row0
+  int32_t col_begin, col_end;   // this slice's columns of the 256-row tile's low-rank operand
+  int32_t grp;                  // first group of that tile
+};
+constexpr int MAX_SEGMENTS = 2;
+
+// Segment number s of rows [m0, m0 + nb) (rows = 0: there is none).
+__host__ __device__ __forceinline__ Segment segment_rows(int m0, int M, int nb, int s) {
+  Segment g = {0, 0, 0, 0, 0, 0};
+  const int end = m0 + nb < M ? m0 + nb : M, t = (m0 >> 8) + s;
+  if (t * 256 >= end) return g;
+  g.row0 = m0 > t * 256 ? m0 : t * 256;
+  g.rows = (end < (t + 1) * 256 ? end : (t + 1) * 256) - g.row0;
+  g.at = g.row0 - m0;
+  return g;
+}
+
+// Arrives on the barrier at this shared-memory offset in both CTAs of the pair (a mask of cluster ranks) once every tcgen05
+// operation issued so far by this thread is done.
+__device__ __forceinline__ void commit_pair(uint32_t bar, uint16_t mask) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"(mask) : "memory");
+}
+
+// 32 rows x 128 columns of accumulators, held one column per lane, as bf16 in the layout of swizzled [rows][64] boxes:
+// neighbouring lanes exchange halves, so that every store is a pair of columns; the lanes of a pair take rows that are four
+// apart, which the swizzle puts into different banks.
+__device__ __forceinline__ void stage_rows(uint32_t buf, const float (&v)[32], int col, int lane) {
+  const bool odd = lane & 1;
+  const uint32_t base = buf + (uint32_t)(col >> 6) * 4096u + (uint32_t)(col & 6) * 2u;
+  const int chunk = (col & 63) >> 3;
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int j = (q >> 2) * 8 + (q & 3);                   // rows j and j + 4
+    const float got = __shfl_xor_sync(0xffffffffu, odd ? v[j] : v[j + 4], 1);
+    const int row = odd ? j + 4 : j;
+    const uint32_t p = odd ? ptx::pack_bf16(got, v[j + 4]) : ptx::pack_bf16(v[j], got);
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(base + (uint32_t)row * 128u + (uint32_t)((chunk ^ (row & 7)) << 4)), "r"(p) : "memory");
+  }
+}
+
+// grid = row tiles x column tiles x slices pairs, clusters of 2 * slices CTAs.
+__global__ void __launch_bounds__(THREADS, 1)
+gemm_masked_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ CUtensorMap tmW,
+                 const __grid_constant__ CUtensorMap tmL, const __grid_constant__ CUtensorMap tmOut,
+                 const __grid_constant__ CUtensorMap tmPbd, const Args args) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES + 2];      // full | empty | accumulator complete | peers' sums
+  __shared__ Segment seg[MAX_SEGMENTS];
+  __shared__ uint32_t keep[9][128];                     // of each 32 rows of the tile: the kept ones, by column
+  __shared__ uint32_t tmem_ptr;
+  __shared__ int abort_word;
+  volatile int* abort_flag = &abort_word;
+  const uint32_t ring = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u, staging = ring + RING_BYTES;
+  const uint32_t bar0 = ptx::smem_u32(bars);
+  auto bar_full = [&](int s) { return bar0 + 8u * s; };
+  auto bar_empty = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
+  const uint32_t bar_done = bar0 + 8u * (2 * MAX_STAGES), bar_sums = bar_done + 8u;
+
+  const int warp = ptx::warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const uint32_t cta = ptx::cluster_ctarank();
+  const uint32_t rank = cta & 1, lead = cta & ~1u;               // CTA of the pair, cluster rank of the pair's leader
+  const bool leader = rank == 0;
+  const int S = args.stages, SK = args.slices, nb = args.nb;
+  const int ks = (int)(cta >> 1);
+  const int tile = (int)blockIdx.x / (2 * SK);
+  const int rt = args.rt0 + tile / args.col_tiles;
+  const int m0 = rt * nb, n0 = tile % args.col_tiles * BN + (int)rank * 128;    // this CTA's columns
+  const uint32_t xhalf = (uint32_t)nb * 64u;                     // this CTA's half of the rows
+  const uint32_t stage = W_BYTES + xhalf;
+  const uint16_t pair_mask = (uint16_t)(3u << lead);
+  constexpr uint32_t tmem_cols = 512;                            // base product [0, 256), low-rank term [256, 512)
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      ptx::mbar_init(bar_full(s), 1);
+      ptx::mbar_init(bar_empty(s), 1);
+    }
+    ptx::mbar_init(bar_done, 1);
+    ptx::mbar_init(bar_sums, 1);
+    abort_word = 0;
+    ptx::fence_barrier_init();
+    ptx::prefetch_tmap(&tmIn);
+    ptx::prefetch_tmap(&tmW);
+    ptx::prefetch_tmap(&tmL);
+    ptx::prefetch_tmap(&tmOut);
+    ptx::prefetch_tmap(&tmPbd);
+  }
+  if (warp == 1) {
+    ptx::tmem2_alloc(ptx::smem_u32(&tmem_ptr), tmem_cols);
+    ptx::tmem2_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::cluster_sync_all();                           // the peers' barriers exist from here on
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = ptx::warp_uniform(tmem_ptr);
+  if (!args.early) ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();
+
+  const int KB = (args.K + GEMM_BK - 1) / GEMM_BK;
+  const int kb_begin = (int)((long long)ks * KB / SK), kb_end = (int)((long long)(ks + 1) * KB / SK);
+  const int box = args.piece_src ? 16 : (args.R < 64 ? args.R : 64);      // rows of an adapter's matrix per low-rank load
+  const int per = 64 / box;
+
+  if (warp == 0) {
+    // ============================ TMA producer (both CTAs) ============================
+    Ring at(S);
+    bool ok = true;
+    const int x_row = m0 + (int)rank * (nb >> 1);
+    for (int kb = kb_begin; kb < kb_end; ++kb, at.next()) {
+      if (!(ok = ptx::warp_all(gemm2_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status)))) break;
+      const uint32_t w = ring + (uint32_t)at.slot * stage, full = ptx::map_to_cta(bar_full(at.slot), lead);
+      if (ptx::elect_one()) {
+        if (leader) ptx::mbar_arrive_expect_tx(bar_full(at.slot), 2 * stage);
+        ptx::tma2_load_2d(w, &tmW, kb * GEMM_BK, n0, full);                               // [N, K]: 128 rows x 64 k
+        ptx::tma2_load_2d(w + W_BYTES, &tmIn, kb * GEMM_BK, x_row, full);
+      }
+    }
+    asm volatile("bar.sync 1, 64;" ::: "memory");                // the segments' table is there
+    // The low-rank operand comes from the launch before; how long that takes must not count against the limit of a wait.
+    if (args.early) ptx::grid_dependency_wait();
+    for (int s = 0; s < MAX_SEGMENTS && ok; ++s) {
+      const Segment g = seg[s];
+      if (g.col_begin >= g.col_end) continue;
+      const int half_rows = ((g.rows + 15) & ~15) >> 1;
+      const int box_begin = g.col_begin / box, box_end = (g.col_end + box - 1) / box;
+      const int pieces = args.piece_src ? args.tile_piece_off[g.row0 >> 8] : 0, per_grp = args.R > 64 ? args.R / 64 : 1;
+      // rows of the adapters' matrices, one box per lane, the next 32 already on their way
+      auto box_rows = [&](int j0) -> int {
+        const int j = j0 + lane;
+        if (j >= box_end) return 0;
+        if (args.piece_src) {
+          const int src = args.piece_src[pieces + j];
+          return (src >> 8) * args.R + (src & 255) * 16;
+        }
+        return args.grp_adapter[g.grp + j / per_grp] * args.R + (j % per_grp) * 64;
+      };
+      const int lc_begin = g.col_begin / 64, n_lc = (g.col_end + 63) / 64 - lc_begin;
+      int batch = (lc_begin * per) & ~31;
+      int cur = box_rows(batch), next = box_rows(batch + 32);
+      for (int i = 0; i < 2 * n_lc; ++i, at.next()) {
+        const bool rest = i >= n_lc;           // all heads, then all remainders: the order does not depend on how a plan packs them
+        const int lc = lc_begin + (rest ? i - n_lc : i), chunk = lc + (rest ? args.rest : 0);
+        if (i == n_lc && batch != ((lc_begin * per) & ~31)) { batch = (lc_begin * per) & ~31; cur = box_rows(batch); next = box_rows(batch + 32); }
+        if (!(ok = ptx::warp_all(gemm2_wait(bar_empty(at.slot), at.parity ^ 1, abort_flag, args.status)))) break;
+        if (((lc * per) & ~31) != batch) { batch += 32; cur = next; next = box_rows(batch + 32); }
+        const int j0 = box_begin > lc * per ? box_begin : lc * per, j1 = box_end < (lc + 1) * per ? box_end : (lc + 1) * per;
+        const int n = box == 8 ? (j1 - j0 + 1) & ~1 : j1 - j0;     // rank 8: a half-filled MMA step repeats the last group (its operand columns are zero)
+        const uint32_t w = ring + (uint32_t)at.slot * stage, full = ptx::map_to_cta(bar_full(at.slot), lead);
+        if (ptx::elect_one()) {
+          if (leader) ptx::mbar_arrive_expect_tx(bar_full(at.slot), 2u * ((uint32_t)(n * box) * 256u + xhalf));
+          // rows of the segment's MMA that this CTA supplies: [half_rows rank, half_rows (rank + 1)) of it (the box may run past them)
+          ptx::tma2_load_2d(w + W_BYTES, &tmPbd, 0, (2 * g.grp + chunk) * 256 + (g.row0 & 255) + (int)rank * half_rows, full);
+        }
+        for (int i2 = 0; i2 < n; ++i2) {     // one box after the other, both 64-column halves: [half][box rows][64]
+          const int brow = __shfl_sync(0xffffffffu, cur, (j0 + i2 < j1 ? j0 + i2 : j1 - 1) & 31);
+          if (ptx::elect_one()) ptx::tma2_load_3d(w + (uint32_t)((j0 + i2 - lc * per) * box) * 256u, &tmL, 0, brow, n0 >> 6, full);
+        }
+      }
+    }
+    // Whoever gives up lets the pair's loads in flight land (the leader's barriers count both CTAs' bytes; bounded: the peer may
+    // not have filled the slot).
+    if (!ok && leader && lane == 0)
+      at.last_uses([&](int slot, uint32_t parity) {
+        for (uint32_t i = 0; i < (1u << 12) && !ptx::mbar_try_wait(bar_full(slot), parity); ++i) {}
+      });
+    __syncwarp();
+  } else if (warp == 1) {
+    // ============================ MMA issuer (leader only) ============================
+    const uint32_t idesc_main = ptx::make_idesc_bf16(256, (uint32_t)nb, false, false);
+    Ring at(S);
+    bool ok = true;
+    // The whole warp walks the loops and one elected lane issues (see gemm2_tcgen05.cuh).
+    if (leader) {
+      uint32_t acc = 0;
+      for (int kb = kb_begin; kb < kb_end; ++kb, at.next()) {
+        if (!(ok = ptx::warp_all(gemm2_wait(bar_full(at.slot), at.parity, abort_flag, args.status)))) break;
+        ptx::tc_fence_after();
+        const uint32_t w = ring + (uint32_t)at.slot * stage;
+        const uint64_t adesc = ptx::make_smem_desc(w, 16, 1024);
+        const uint64_t bdesc = ptx::make_smem_desc(w + W_BYTES, 16, 1024);
+        if (ptx::elect_one()) {
+#pragma unroll
+          for (int k = 0; k < GEMM_BK / 16; ++k)
+            ptx::umma2_f16(tmem_base, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc_main, k == 0 ? acc : 1u);
+          commit_pair(bar_empty(at.slot), pair_mask);
+        }
+        acc = 1;
+      }
+    }
+    __syncwarp();
+    asm volatile("bar.sync 3, 64;" ::: "memory");
+    if (leader) {
+      if (args.early) ptx::grid_dependency_wait();                // as the producer
+      // boxes of [2 halves][BOX rows][64 columns]: 16 operand columns are 16 rows of one box, or two boxes of 8
+      auto lora_mma = [&](auto box_rows) {
+        constexpr int BOX = decltype(box_rows)::value;
+        for (int s = 0; s < MAX_SEGMENTS && ok; ++s) {
+          const Segment g = seg[s];
+          if (g.col_begin >= g.col_end) continue;
+          const uint32_t idesc = ptx::make_idesc_bf16(256, (uint32_t)((g.rows + 15) & ~15), true, false);
+          const uint32_t d = tmem_base + (uint32_t)(256 + g.at);
+          const int lc_begin = g.col_begin / 64, n_lc = (g.col_end + 63) / 64 - lc_begin;
+          uint32_t acc = 0;
+          for (int i = 0; i < 2 * n_lc; ++i, at.next()) {
+            const int lc = lc_begin + (i >= n_lc ? i - n_lc : i);
+            if (!(ok = ptx::warp_all(gemm2_wait(bar_full(at.slot), at.parity, abort_flag, args.status)))) break;
+            ptx::tc_fence_after();
+            const uint32_t w = ring + (uint32_t)at.slot * stage;
+            const uint64_t adesc = ptx::make_smem_desc(w, BOX * 128, BOX == 8 ? 2048 : 1024);
+            const uint64_t bdesc = ptx::make_smem_desc(w + W_BYTES, 16, 1024);
+            const int from = g.col_begin - lc * 64, to = g.col_end - lc * 64;
+            if (ptx::elect_one()) {
+#pragma unroll
+              for (int k = 0; k < GEMM_BK / 16; ++k)
+                if (k * 16 >= from && k * 16 < to) {
+                  constexpr int per_box = BOX < 16 ? 1 : BOX / 16;
+                  const uint32_t at_k = BOX == 8 ? k * 4096 : (k / per_box) * BOX * 256 + (k % per_box) * 2048;
+                  ptx::umma2_f16(d, adesc + (uint64_t)(at_k >> 4), bdesc + (uint64_t)(k * 2), idesc, acc);
+                  acc = 1;
+                }
+              commit_pair(bar_empty(at.slot), pair_mask);
+            }
+            acc = 1;
+          }
+        }
+      };
+      if (box == 8) lora_mma(std::integral_constant<int, 8>());
+      else if (box == 16) lora_mma(std::integral_constant<int, 16>());
+      else if (box == 32) lora_mma(std::integral_constant<int, 32>());
+      else lora_mma(std::integral_constant<int, 64>());
+      if (ok && ptx::elect_one()) commit_pair(bar_done, pair_mask);
+    }
+    __syncwarp();
+  } else {
+    // ============================ low-rank tables (plan data: not written by any kernel) ============================
+    if (warp == 2) {
+      if (lane < MAX_SEGMENTS) {
+        Segment g = segment_rows(m0, args.M, nb, lane);
+        if (g.rows > 0) {
+          const int t = g.row0 >> 8;
+          g.grp = args.tile_grp_off[t];
+          const int n_grp = args.tile_grp_off[t + 1] - g.grp;
+          // A slice takes whole adapter groups, the same ones however wide a plan packs them.
+          int gb = (int)((long long)ks * n_grp / SK), ge = (int)((long long)(ks + 1) * n_grp / SK);
+          if (args.R == 8) { gb &= ~1; if (ks + 1 < SK) ge &= ~1; }
+          auto column = [&](int gi) { return !args.tile_cols ? gi * args.R : (gi < n_grp ? args.grp_col[g.grp + gi] : args.tile_cols[t]); };
+          g.col_begin = column(gb);
+          g.col_end = column(ge);
+        }
+        seg[lane] = g;
+      }
+      __syncwarp();
+      asm volatile("bar.arrive 1, 64;\n\tbar.arrive 3, 64;" ::: "memory");
+    }
+    asm volatile("bar.sync 2, 128;" ::: "memory");             // all four warps read the segments' table later
+    // keep decisions of this lane's column, 32 rows to a word; the four lanes of a group of four columns share their generator's
+    // outputs: each computes every fourth row's
+    const int col = (warp & 3) * 32 + lane, f = lane & 3;
+    for (int j0 = 0; j0 < nb; j0 += 32) {
+      uint32_t bits = 0;
+      for (int j = 0; j < 32; j += 4) {
+        const uint64_t z = drop_bits(args.drop.seed, (uint32_t)(m0 + j0 + j + f), (uint32_t)((n0 + col) >> 2));
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const uint32_t z0 = __shfl_sync(0xffffffffu, (uint32_t)z, (lane & ~3) | r), z1 = __shfl_sync(0xffffffffu, (uint32_t)(z >> 32), (lane & ~3) | r);
+          const uint32_t w = f & 2 ? z1 : z0, field = f & 1 ? w >> 16 : w & 0xFFFFu;
+          bits |= (field >= args.drop.thr ? 1u : 0u) << (j + r);
+        }
+      }
+      keep[j0 >> 5][col] = bits;
+    }
+    // The MMAs of the low-rank blocks wait for the launch before, so its time must not count against the limit of the wait
+    // here.  And no CTA stores or ends before that launch has ended: what follows in the stream may rely on that.
+    ptx::grid_dependency_wait();
+    gemm2_wait(bar_done, 0, abort_flag, args.status);
+    ptx::tc_fence_after();
+  }
+  __syncwarp();
+
+  // ============================ the slices' sums, the result ============================
+  // Every CTA of a cut tile is done with its ring (its pair's MMAs have completed, or it gave up and its loads have landed), so
+  // the rings take the fp32 sums: slice d finishes rows [d chunk, (d + 1) chunk) of the tile.  Each CTA lays the rows that its
+  // peers finish out as [row][128] and sends them as one bulk copy each; what arrives lands as [slice][row][128] behind
+  // them, and is added to the accumulator's own part in slice order.
+  if (SK > 1) {
+    __syncthreads();
+    ptx::cluster_sync_all();
+  }
+  if (warp >= 2) {
+    const int e = warp & 3, col = e * 32 + lane;
+    const uint32_t taddr = tmem_base + ((uint32_t)(e * 32) << 16);
+    const int chunk = slice_rows(nb, SK);
+    // this lane's column of rows [j0, j0 + 32) of the tile (what lies past its end is not used)
+    auto load_rows = [&](int j0, float (&v)[32]) {
+      uint32_t u[32];
+      ptx::tmem_ld_32x32b_x32(taddr + (uint32_t)j0, u);
+      ptx::tmem_ld_wait();
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(u[j]);
+      uint32_t bits = 0;                           // kept rows, of those that this slice has low-rank blocks of
+      for (int s = 0; s < MAX_SEGMENTS; ++s)
+        if (seg[s].col_begin < seg[s].col_end) {
+          const int from = seg[s].at, to = seg[s].at + seg[s].rows;
+          if (j0 >= from && j0 < to) bits |= 0xFFFFu;
+          if (j0 + 16 >= from && j0 + 16 < to) bits |= 0xFFFF0000u;
+        }
+      if (bits != 0) {
+        bits &= j0 & 16 ? __funnelshift_r(keep[j0 >> 5][col], keep[(j0 >> 5) + 1][col], 16) : keep[j0 >> 5][col];     // j0 is a multiple of 16
+        ptx::tmem_ld_32x32b_x32(taddr + 256u + (uint32_t)j0, u);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] += (bits >> j) & 1u ? __uint_as_float(u[j]) * args.drop.keep_scale : 0.f;
+      }
+    };
+    const uint32_t part = (uint32_t)chunk * 512u, arrived = ring + (uint32_t)(SK - 1) * part;
+    if (SK > 1) {
+      for (int i = 1; i < SK; ++i) {
+        const int d = ks + i < SK ? ks + i : ks + i - SK;
+        const uint32_t out = ring + (uint32_t)(i - 1) * part + (uint32_t)col * 4u;
+        for (int j0 = 0; j0 < chunk && d * chunk + j0 < nb; j0 += 32) {
+          float v[32];
+          load_rows(d * chunk + j0, v);
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (j < 16 || j0 + 16 < chunk) asm volatile("st.shared.f32 [%0], %1;" ::"r"(out + (uint32_t)(j0 + j) * 512u), "f"(v[j]) : "memory");
+        }
+      }
+      ptx::fence_proxy_async_smem();
+      asm volatile("bar.sync 2, 128;" ::: "memory");
+      if (threadIdx.x == 64) {
+        ptx::mbar_arrive_expect_tx(bar_sums, (uint32_t)(SK - 1) * part);
+        for (int i = 1; i < SK; ++i) {
+          const uint32_t d = (uint32_t)(ks + i < SK ? ks + i : ks + i - SK);
+          rows::bulk_to_cta(ptx::map_to_cta(arrived + (uint32_t)(SK - 1 - i) * part, 2 * d + rank), ring + (uint32_t)(i - 1) * part, part,
+                            ptx::map_to_cta(bar_sums, 2 * d + rank));
+        }
+      }
+      gemm_wait(bar_sums, 0, abort_flag, args.status);
+    }
+    const bool good = *abort_flag == 0;
+    uint32_t buf = staging;
+    const int first = ks * chunk, last = nb < first + chunk ? nb : first + chunk;
+    for (int j0 = first; j0 < last && m0 + j0 < args.M; j0 += 32, buf ^= 8192u) {
+      float v[32];
+      load_rows(j0, v);
+      if (SK > 1) {
+        // the slices in order: those before this CTA's own, its own, those behind it
+        float own[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) { own[j] = v[j]; v[j] = 0.f; }
+        for (int s = 0; s < SK; ++s) {
+          const int i = s - ks + (s < ks ? SK : 0);                // arrival slot i - 1
+          const uint32_t from = arrived + (uint32_t)(i - 1) * part + (uint32_t)(j0 - first) * 512u + (uint32_t)col * 4u;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            float x = own[j];
+            if (s != ks) asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(from + (uint32_t)j * 512u) : "memory");
+            v[j] += x;
+          }
+        }
+      }
+      if (threadIdx.x == 64) ptx::tma_store_wait_read<1>();       // the buffer's last stores have been read
+      asm volatile("bar.sync 2, 128;" ::: "memory");
+      stage_rows(buf, v, col, lane);
+      ptx::fence_proxy_async_smem();
+      asm volatile("bar.sync 2, 128;" ::: "memory");
+      if (threadIdx.x == 64) {
+        for (int c = 0; c < 2 && good; ++c)                       // boxes of 64 columns x 16 rows
+          if (n0 + c * 64 < args.N) {
+            ptx::tma_store_2d(&tmOut, buf + (uint32_t)c * 4096u, n0 + c * 64, m0 + j0);
+            if (j0 + 16 < last && m0 + j0 + 16 < args.M)
+              ptx::tma_store_2d(&tmOut, buf + (uint32_t)c * 4096u + 2048u, n0 + c * 64, m0 + j0 + 16);
+          }
+        ptx::tma_store_commit();
+      }
+    }
+    if (threadIdx.x == 64) ptx::tma_store_wait<0>();
+    __syncwarp();
+  }
+
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::cluster_sync_all();          // the peers are done with this CTA's shared memory and barriers
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    ptx::tmem2_dealloc(tmem_base, tmem_cols);
+  }
+}
+
+}  // namespace masked
+}  // namespace mlora

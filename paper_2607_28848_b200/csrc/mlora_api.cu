@@ -20,6 +20,7 @@
 #include "gemm_tcgen05.cuh"
 #include "gemm2_tcgen05.cuh"
 #include "gemm_rows_tcgen05.cuh"
+#include "gemm_masked_tcgen05.cuh"
 #include "simt.cuh"
 #include "skinny.cuh"
 #include "grad_tc.cuh"
@@ -443,6 +444,62 @@ int lowrank_columns(const RowSpace& hs, int R) {
     most = n > most ? n : most;
   }
   return most * R;
+}
+
+// Clusters of 1 to 4 pairs of the masked input-gradient kernel that are resident at once (nullptr: the query failed).
+const int* masked_clusters(const mlora_ctx* ctx) {
+  static int clusters_dev[kMaxDevices][5] = {};
+  int* clusters = clusters_dev[ctx->device];
+  std::lock_guard<std::mutex> lock(g_attr_mutex);
+  if (clusters[1] > 0) return clusters;
+  if (cudaFuncSetAttribute(masked::gemm_masked_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)masked::SMEM_BYTES) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+  for (int c = 4; c >= 1; --c) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctx->sm_count / (2 * c) * 2 * c); cfg.blockDim = dim3(masked::THREADS); cfg.dynamicSmemBytes = masked::SMEM_BYTES;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2 * c; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, masked::gemm_masked_kernel, &cfg) != cudaSuccess || n <= 0) { cudaGetLastError(); return nullptr; }
+    clusters[c] = n;
+  }
+  return clusters;
+}
+
+// Rows of a tile, K slices and the row tiles of a launch of the masked input gradient, or false: the product and the masked expand in
+// launches of their own (kernel variants, and outputs wider than the pairs).  Costs in us as fitted to 925 calls (65 to 1600 rows, ranks 8
+// to 128, 142 shapes) with each tile height and slice count forced in turn.  Whole backward calls, product and masked expand in
+// launches of their own / here, us: 222 rows 3328 -> 8448 rank 16 67.2 / 38.1, 566 rows 4032 -> 3136 rank 32 103.9 / 53.8, 1277 rows
+// 2240 -> 4864 rank 8 68.1 / 64.4, 1477 rows 2368 -> 13888 rank 64 312 / 195, 163 rows 1280 -> 2816 rank 128 151 / 36; of 36 drawn calls of
+// 36 to 3432 rows none was slower.
+struct MaskedShape { int nb, slices, row_tiles; };
+bool masked_shape(const mlora_ctx* ctx, int M, int N, int K, int lr_cols, MaskedShape& w) {
+  if (ctx->gemm_path != 0 || ctx->shrink_path != 0 || !ctx->gemm_pairs || ctx->no_split_k || ctx->grad_mode != 0) return false;
+  const int* clusters = masked_clusters(ctx);
+  if (!clusters) return false;
+  const int kblocks = K / GEMM_BK, lc = 2 * ((lr_cols + 63) / 64), cols = (N + masked::BN - 1) / masked::BN;
+  float best = 1e30f;
+  for (int sk = 1; sk <= 4 && (sk == 1 || kblocks >= 8 * sk); ++sk) {
+    const int rt_most = clusters[sk] / cols;
+    if (rt_most < 1) break;
+    for (int launches = 1; launches <= (M + 255) / 256; ++launches) {
+      for (int aligned = 0; aligned < 2; ++aligned) {
+        int nb = ((M + rt_most * launches - 1) / (rt_most * launches) + 15) / 16 * 16;
+        if (aligned) { int p = 32; while (p < nb) p *= 2; nb = p; }      // no tile straddles two 256-row tiles of the low-rank operand
+        if (nb < 32) nb = 32;
+        if (nb > 256) continue;
+        const int segs = 256 % nb == 0 || M <= 256 ? 1 : 2, chunk = masked::slice_rows(nb, sk);
+        const float block = fmaxf(0.18f, 0.235f + 0.154f * (nb / 256.f));
+        float cost = 4.4f + (float)((kblocks + sk - 1) / sk) * block + (float)(segs * lc) / sk * 0.28f + chunk * 0.003f;
+        if (sk > 1) cost += 3.3f + (sk - 1) * chunk * 0.027f;
+        cost *= launches;
+        if (cost < best) { best = cost; w = {nb, sk, rt_most}; }
+      }
+      if (best < 1e29f && launches * rt_most * 32 >= M) break;
+    }
+  }
+  return best < 1e29f;
 }
 
 // CTAs along K per item of the few-row shrink: with the items, as many as two per SM.
@@ -1104,6 +1161,40 @@ mlora_status_t launch_gemm_rows(mlora_ctx* ctx, const mlora_layer_t* L, const Ro
   return scope.done();
 }
 
+// dX under dropout: W read as the transposed operand, one launch per wave of row tiles.
+mlora_status_t launch_gemm_masked(mlora_ctx* ctx, const mlora_layer_t* L, const RowSpace& hs, const DevRowSpace& ds, const void* dY,
+                                  int64_t lddy, void* dX, int64_t lddx, int M, const MaskedShape& shape, cudaStream_t st) {
+  const int R = L->rank, N = L->d_in, K = L->d_out, nb = shape.nb;
+  const uint64_t groups = hs.grp2_adapter.size();
+  const bool ranked = ds.piece_src != nullptr;
+  masked::Args a;
+  a.M = M; a.N = N; a.K = K; a.R = R; a.nb = nb; a.slices = shape.slices;
+  a.early = 1;                                       // behind this call's gradient kernel
+  a.tile_grp_off = ds.tile2_grp_off; a.grp_adapter = ds.grp2_adapter;
+  a.tile_cols = ranked ? ds.tile2_cols : nullptr; a.grp_col = ds.grp2_col; a.tile_piece_off = ds.tile2_piece_off; a.piece_src = ranked ? ds.piece_src : nullptr;
+  a.drop = ctx->drop; a.rest = 2 * (int)groups; a.status = ctx->status_dev;
+  a.col_tiles = (N + masked::BN - 1) / masked::BN;
+  a.stages = (int)(masked::RING_BYTES / masked::stage_bytes(nb));
+  a.stages = a.stages < masked::MAX_STAGES ? a.stages : masked::MAX_STAGES;
+  CUtensorMap tIn, tW, tL, tOut, tPbd;
+  mlora_status_t s;
+  if ((s = make_tmap_bf16(ctx, &tIn, dY, K, M, lddy, GEMM_BK, nb / 2)) != MLORA_OK) return s;
+  if ((s = make_tmap_bf16(ctx, &tW, L->W, K, N, L->ldw, GEMM_BK, 128)) != MLORA_OK) return s;
+  if ((s = make_tmap_bf16(ctx, &tOut, dX, N, M, lddx, 64, 16)) != MLORA_OK) return s;
+  if ((s = make_tmap_bf16_blocked(ctx, &tL, L->A_all, (uint64_t)L->n_adapters * R, N, N, ranked ? 16 : (R < 64 ? R : 64), 2)) != MLORA_OK) return s;
+  if ((s = make_tmap_bf16(ctx, &tPbd, ctx->ws_pbd, 64, groups * 1024, 64, 64, nb / 2)) != MLORA_OK) return s;
+  const int row_tiles = (M + nb - 1) / nb;
+  for (a.rt0 = 0; a.rt0 < row_tiles; a.rt0 += shape.row_tiles) {
+    const int tiles = a.col_tiles * std::min(row_tiles - a.rt0, shape.row_tiles);
+    if (cancelled(ctx)) return MLORA_CANCELLED;
+    LaunchScope scope(ctx, st, KIND_GEMM_BWD);
+    launch_pdl_cluster(scope.slot < 0, masked::gemm_masked_kernel, dim3(tiles * 2 * a.slices), dim3(masked::THREADS), dim3(2 * a.slices, 1, 1),
+                       masked::SMEM_BYTES, st, tIn, tW, tL, tOut, tPbd, a);
+    if ((s = scope.done()) != MLORA_OK) return s;
+  }
+  return MLORA_OK;
+}
+
 // Out = In Wop + (scale) P L over one row space, tensor-core path.  `early`: the launch in front of this one in the stream
 // is this call's own rank-r or gradient kernel (see gemm_rows_tcgen05.cuh).
 template <bool W_KMAJOR>
@@ -1680,8 +1771,8 @@ mlora_status_t grow_workspaces(mlora_ctx* ctx, const HostPlan& h, int32_t n_rows
     if ((s = replace_workspace(ctx, (void**)&ctx->ws_pop, (size_t)nb * 2 * 65536, false)) != MLORA_OK) return s;
     ctx->ws_pop_blocks = nb;
   }
-  const int64_t groups = (int64_t)(h.fwd.grp2_adapter.size() > h.bwd.grp2_adapter.size() ? h.fwd.grp2_adapter.size()
-                                                                                        : h.bwd.grp2_adapter.size());
+  // (the fine-tuning rows' twice: under dropout the input gradient takes their values' remainders as well)
+  const int64_t groups = (int64_t)std::max(h.fwd.grp2_adapter.size(), 2 * h.bwd.grp2_adapter.size());
   if (groups > ctx->ws_pbd_groups) {   // two chunk slots of [256][64] bf16 per adapter group of a tile
     const int64_t g = grown(groups, ctx->ws_pbd_groups);
     if ((s = replace_workspace(ctx, (void**)&ctx->ws_pbd, (size_t)g * 2 * 256 * 64 * sizeof(__nv_bfloat16), false)) != MLORA_OK) return s;
@@ -1908,8 +1999,11 @@ mlora_status_t mlora_backward(mlora_ctx* ctx, const mlora_layer_t* L, const mlor
   sa.In = (const __nv_bfloat16*)dY; sa.ld_in = lddy; sa.D = L->d_out;
   sa.P_all = (const __nv_bfloat16*)L->B_all; sa.scale = L->scale; sa.Out = ctx->ws_p;
   sa.item_rows = p->bwd.item_rows; sa.item_start = p->bwd.item_start; sa.item_nrows = p->bwd.item_nrows;
-  sa.pbd = PbdArgs{(ctx->gemm_pairs && dX && !dropping) ? ctx->ws_pbd : nullptr, p->bwd.row_grp2, p->bwd.tile2_grp_off, nullptr,
+  MaskedShape mshape;
+  const bool masked = dropping && dX && masked_shape(ctx, h.ft_rows, L->d_in, L->d_out, lowrank_columns(h.bwd, L->rank), mshape);
+  sa.pbd = PbdArgs{(ctx->gemm_pairs && dX && (!dropping || masked)) ? ctx->ws_pbd : nullptr, p->bwd.row_grp2, p->bwd.tile2_grp_off, nullptr,
                    p->bwd.zero_rows2, (int32_t)h.bwd.zero_rows2.size()};
+  sa.pbd.remainder = masked ? 2 * (int)h.bwd.grp2_adapter.size() : 0;      // behind the operand itself: two slots per group
   set_ranked(sa.pbd, p->bwd);
   sa.item_adapter = p->bwd.item_adapter; sa.item_save = nullptr; sa.x_save = nullptr; sa.u_save = nullptr; sa.save_base = 0; sa.save_cap = 0;
   // V on the tcgen05 shrink from rank kTcShrinkMinRank (every rank under kernel variant 6), else on the mma.sync kernels
@@ -1965,6 +2059,7 @@ mlora_status_t mlora_backward(mlora_ctx* ctx, const mlora_layer_t* L, const mlor
                         : launch_grad_stream2<4>(ctx, p, ga, gA, n_slots, h.ft_rows, st);
     if (s != MLORA_OK) return s;
     if (!dX) return MLORA_OK;
+    if (masked) return launch_gemm_masked(ctx, L, h.bwd, p->bwd, dY, lddy, dX, lddx, h.ft_rows, mshape, st);
     if (dropping) {   // the mask acts on the low-rank term per element: base product first, then the masked expand
       if ((s = gemm_bf16<true>(ctx, L, h.bwd, p->bwd, dY, lddy, dX, lddx, L->A_all, ctx->ws_p, nullptr, h.ft_rows,
                                L->d_in, L->d_out, st, true, false)) != MLORA_OK)
@@ -1980,6 +2075,7 @@ mlora_status_t mlora_backward(mlora_ctx* ctx, const mlora_layer_t* L, const mlor
   if (dropping) ga.drop = ctx->drop;
   if ((s = launch_grad(ctx, p, ga, n_slots, h.ft_rows, st)) != MLORA_OK) return s;
   if (!dX) return MLORA_OK;
+  if (masked) return launch_gemm_masked(ctx, L, h.bwd, p->bwd, dY, lddy, dX, lddx, h.ft_rows, mshape, st);
   if (dropping) {   // the mask acts on the low-rank term per element: base product first, then the masked expand
     if ((s = gemm_bf16<true>(ctx, L, h.bwd, p->bwd, dY, lddy, dX, lddx, L->A_all, ctx->ws_p, nullptr, h.ft_rows, L->d_in,
                              L->d_out, st, true, false)) != MLORA_OK)

@@ -1,0 +1,57 @@
+"""The input gradient under dropout where its row tiles, segments and K slices can go wrong: heights that are no multiple of 32, tiles
+that straddle the 256-row tiles of the low-rank operand, column tiles that are half empty, one to four slices (whose shares of a
+tile's rows start at any multiple of 16), several launches, every rank, plans with ranks of their own."""
+import numpy as np
+import pytest
+
+from paper_2607_28848_b200 import binding as mb
+from paper_2607_28848_b200 import synth
+from paper_2607_28848_b200.runner import LayerRun, Session
+from test_gpu_variants import check_dropout
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sess():
+    s = Session(0)
+    yield s
+    s.close()
+
+
+@pytest.mark.parametrize("rank", [8, 16, 32, 64, 128])
+@pytest.mark.parametrize("rows,d_in,d_out", [(20, 320, 192), (130, 448, 1088), (250, 1344, 6400), (700, 1344, 1024), (1300, 4096, 256)])
+def test_parity(sess, rows, d_in, d_out, rank):
+    w = synth.random_workload(2200 + rows + rank, d_in, d_out, rank, 4, rows, max_seg=max(2, rows // 2), p_finetune=0.8)
+    check_dropout(sess, w, synth.make_tensors(w), 0.2, 2 ** 35 + rows, blocked=True)
+
+
+def test_every_row_its_own_adapter(sess):
+    """An odd number of groups in every slice, many more low-rank blocks than main ones."""
+    segs = synth.segments_array([(i, 1, (7 * i) % 131, 1) for i in range(120)] + [(120, 30, 5, 1)])
+    w = synth.Workload("own_adapters", 512, 1024, 8, 131, "bf16", 150, segs, seed=8)
+    check_dropout(sess, w, synth.make_tensors(w), 0.1, 99, blocked=True)
+
+
+@pytest.mark.parametrize("rows,d_in,d_out", [(600, 1024, 320), (300, 256, 4096)])
+def test_plans_with_ranks_of_their_own(sess, rows, d_in, d_out):
+    """The padded plan's bits, whichever way the operand is packed."""
+    ranks = [16, 64, 32, 8]
+    w = synth.random_workload(2300, d_in, d_out, 64, len(ranks), rows, max_seg=150, p_finetune=0.9)
+    t = synth.make_tensors(w)
+    for a, r in enumerate(ranks):
+        t["A_all"][a, r:] = 0
+        t["B_all"][a, r:] = 0
+    outs = []
+    mb.mlora_set_dropout(sess.ctx, 0.1, 77)
+    try:
+        for ar in (None, ranks):
+            run = LayerRun(sess, w.dtype, t, w.segments, w.n_rows, adapter_rank=ar)
+            run.forward()
+            run.backward()
+            assert run.status() == mb.MLORA_OK
+            outs.append(run.host(run.dX))
+            run.close()
+    finally:
+        mb.mlora_set_dropout(sess.ctx, 0.0, 0)
+    assert np.array_equal(*outs)
